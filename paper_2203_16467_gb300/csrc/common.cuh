@@ -43,13 +43,15 @@ struct Ctrl {
     double sumE;            // sum of E
     // mechanics
     double mech_target, R2, rr, pAp, rAp, qq, alpha, beta, cg_target;
+    double rr_inv;          // 1 / rr (0 for rr = 0), formed beside alpha
     int nd_a, nd_b, newton_it, needs_fold;
     int cg_a, cg_b, cg_it, cg_total, cg_break;
     // near-equilibrium rescale (Algorithm 4 lines 4-10)
     double mF_max, D_max, Rf_star, D_star, gamma;
     int istar, flag, rescaled;
     // phase field (Algorithm 1)
-    double pf_rr, pf_rp, pJp, pf_alpha, pf_beta, pf_target, pf_best;
+    double pf_rr, pf_rp, pJp, pf_alpha, pf_beta, pf_target, pf_best;   // pf_best, pf_last_full: squared norms
+    double pf_irp;          // -1 / (r.p) of the direction, formed beside alpha
     double pf_pap;          // sum a p^2 of the direction (the diagonal part of p.Jp)
     int pf_a, pf_b, pf_it, pf_break, n_active, pf_best_it, pf_clamp_iters;
     // residual recurrence: pf_full = this iteration evaluates Jv explicitly

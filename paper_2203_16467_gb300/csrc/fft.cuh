@@ -77,7 +77,7 @@ __device__ __forceinline__ void dft8(C (&u)[8]) {
 // TWP: the twiddle table is stored with padded indices (pidx), as when staged in
 // shared memory, so that the strided reads of a warp spread over the banks.
 template <typename T, int M, int R, int G, int NSEQ, int SP, int NT, bool INV, bool TWP = false>
-__device__ __forceinline__ void stockham_pass(typename CT<T>::t* buf, int s0, int p, const typename CT<T>::t* tw) {
+__device__ __forceinline__ void stockham_pass(typename CT<T>::t* buf, int s0, int p, const typename CT<T>::t* tw, int tid) {
     using C = typename CT<T>::t;
     constexpr int NBS = M / R;           // butterflies per sequence
     constexpr int NB = G * NBS;          // butterflies in the round
@@ -85,7 +85,7 @@ __device__ __forceinline__ void stockham_pass(typename CT<T>::t* buf, int s0, in
     C u[PER][8];
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
-        int b = threadIdx.x + j * NT;
+        int b = tid + j * NT;
         int s = s0 + b / NBS, i = b % NBS;
         if ((NB % NT == 0 || b < NB) && s < NSEQ) {
 #pragma unroll
@@ -95,7 +95,7 @@ __device__ __forceinline__ void stockham_pass(typename CT<T>::t* buf, int s0, in
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
-        int b = threadIdx.x + j * NT;
+        int b = tid + j * NT;
         int s = s0 + b / NBS, i = b % NBS;
         if ((NB % NT == 0 || b < NB) && s < NSEQ) {
             const int k = i & (p - 1);
@@ -144,20 +144,20 @@ __device__ __forceinline__ void stockham_pass(typename CT<T>::t* buf, int s0, in
 // of 3.  Sequences are processed in rounds of G; each thread holds at most PER8
 // radix-8 butterflies of a round in registers.
 template <typename T, int M, int NSEQ, int SP, int NT, bool INV, bool TWP = false>
-__device__ __forceinline__ void fft_smem(typename CT<T>::t* buf, const typename CT<T>::t* tw) {
+__device__ __forceinline__ void fft_smem(typename CT<T>::t* buf, const typename CT<T>::t* tw, int tid = threadIdx.x) {
     constexpr int LOG = ilog2(M);
     constexpr int PER8 = sizeof(T) == 4 ? 2 : 1;
     constexpr int G = cmax(1, cmin(NSEQ, (8 * NT * PER8) / M));   // sequences per round
     for (int s0 = 0; s0 < NSEQ; s0 += G) {
         int p = 1;
         if (LOG % 3 == 1) {
-            stockham_pass<T, M, 2, G, NSEQ, SP, NT, INV, TWP>(buf, s0, 1, tw);
+            stockham_pass<T, M, 2, G, NSEQ, SP, NT, INV, TWP>(buf, s0, 1, tw, tid);
             p = 2;
         } else if (LOG % 3 == 2) {
-            stockham_pass<T, M, 4, G, NSEQ, SP, NT, INV, TWP>(buf, s0, 1, tw);
+            stockham_pass<T, M, 4, G, NSEQ, SP, NT, INV, TWP>(buf, s0, 1, tw, tid);
             p = 4;
         }
-        for (; p < M; p *= 8) stockham_pass<T, M, 8, G, NSEQ, SP, NT, INV, TWP>(buf, s0, p, tw);
+        for (; p < M; p *= 8) stockham_pass<T, M, 8, G, NSEQ, SP, NT, INV, TWP>(buf, s0, p, tw, tid);
     }
 }
 
@@ -433,34 +433,26 @@ __device__ __forceinline__ void row_inv_item(const Desc<T>& d, const typename F:
     }
     cp_async_wait_all();
     __syncthreads();
+    // (a lane's two values replace the two that it read, so the combination runs in place)
     constexpr int H = M / 2, NI = (Cfg::NSEQ * H + NT - 1) / NT;
-    C z[NI][2];
 #pragma unroll
     for (int u = 0; u < NI; ++u) {
         const int t = threadIdx.x + u * NT;
         if ((Cfg::NSEQ * H) % NT == 0 || t < Cfg::NSEQ * H) {
             const int s = t / H, k = t % H;
-            C xk = buf[s * SP + pidx(k)], xm = buf[s * SP + pidx(M - k)];
+            C *lo = &buf[s * SP + pidx(k)], *hi = &buf[s * SP + pidx(M - k)];
+            C xk = *lo, xm = *hi;
             if (k == 0) { xk.y = T(0); xm.y = T(0); }
             xm.y = -xm.y;
             C A = cadd(xk, xm);
             C B = cmulc(csub(xk, xm), twN[k]);
-            z[u][0] = C{A.x - B.y, A.y + B.x};
-            z[u][1] = C{A.x + B.y, B.x - A.y};
-            if (k == 0) {
-                const C xh = buf[s * SP + pidx(H)];
-                z[u][1] = C{T(2) * xh.x, T(-2) * xh.y};
+            *lo = C{A.x - B.y, A.y + B.x};
+            if (k > 0) {
+                *hi = C{A.x + B.y, B.x - A.y};
+            } else {
+                C* h = &buf[s * SP + pidx(H)];
+                *h = C{T(2) * h->x, T(-2) * h->y};
             }
-        }
-    }
-    __syncthreads();
-#pragma unroll
-    for (int u = 0; u < NI; ++u) {
-        const int t = threadIdx.x + u * NT;
-        if ((Cfg::NSEQ * H) % NT == 0 || t < Cfg::NSEQ * H) {
-            const int s = t / H, k = t % H;
-            buf[s * SP + pidx(k)] = z[u][0];
-            buf[s * SP + pidx(k == 0 ? H : M - k)] = z[u][1];
         }
     }
     __syncthreads();

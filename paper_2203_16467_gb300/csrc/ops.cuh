@@ -216,6 +216,9 @@ struct FCgIn {
             c->cg_b = 1;
         } else {
             c->alpha = c->rr / pAp;
+            // for FCgOut's beta, whose finalizer ends the iteration's chain (an FP64 division takes
+            // 550 cycles, a square root 600, a product 65)
+            c->rr_inv = c->rr > 0.0 ? 1.0 / c->rr : 0.0;
         }
     }
 };
@@ -252,12 +255,12 @@ struct FCgOut {
     }
     __device__ static void finalize(const Desc<T>& d, const double* tot) {
         Ctrl* c = d.ctrl;
-        const double rr = tot[0], rr_old = c->rr;
+        const double rr = tot[0];
         c->cg_it += 1;
         c->cg_total += 1;
-        c->beta = rr_old > 0.0 ? rr / rr_old : 0.0;
+        c->beta = rr * c->rr_inv;
         c->rr = rr;
-        const bool conv = sqrt(rr) <= c->cg_target;
+        const bool conv = rr <= c->cg_target * c->cg_target;
         if (conv || c->cg_it >= d.k.max_cg) {
             if (!conv) c->status |= 1;
             c->cg_b = 1;
@@ -462,8 +465,8 @@ struct FPfInit {
         c->pf_rp = -tot[0];
         c->bar_count = 0;
         c->bar_abort = 0;
-        c->pf_last_full = rn;
-        c->pf_best = rn;
+        c->pf_last_full = tot[0];
+        c->pf_best = tot[0];
         c->pf_best_it = 0;
         int done = rn <= target;
         c->pf_a = done;
@@ -605,6 +608,7 @@ struct FPfA3 {   // J p; p.Jp, r.p -> alpha = -(r.p)/(p.Jp)
         Ctrl* c = d.ctrl;
         c->pJp = tot[0];
         c->pf_rp = tot[1];
+        c->pf_irp = tot[1] != 0.0 ? -1.0 / tot[1] : 0.0;
         if (!(tot[0] > 0.0)) {
             c->pf_break = 1;
             c->pf_alpha = 0.0;
@@ -653,6 +657,7 @@ struct FColLapPFQ {
         } else {
             c->pf_alpha = -c->pf_rp / pJp;
         }
+        c->pf_irp = c->pf_rp != 0.0 ? -1.0 / c->pf_rp : 0.0;   // for the beta of this iteration
     }
 };
 
@@ -667,27 +672,26 @@ __device__ __forceinline__ void pf_next_dir(Ctrl* c, const double* S) {
 // explicit residual kernel: beta, ||r||, active count and the stopping decision.
 template <typename T>
 __device__ __forceinline__ void pf_finish(const Desc<T>& d, Ctrl* c, double rr, double rro, double nact, bool full) {
-    if (!d.k.pf_precond) {   // (the preconditioned variant takes beta from the z pass)
-        double den = -c->pf_rp;   // = alpha p.Jp
-        c->pf_beta = den != 0.0 ? (rr - rro) / den : 0.0;
-    }
+    // (the preconditioned variant takes beta from the z pass); -r.p = alpha p.Jp
+    if (!d.k.pf_precond) c->pf_beta = (rr - rro) * c->pf_irp;
     c->pf_rr = rr;
     c->pf_it += 1;
     c->n_active = (int)nact;
-    double rn = sqrt(rr);
+    // norms are compared by their squares (no square root on the iteration's chain)
+    const double target2 = c->pf_target * c->pf_target;
     bool conv = false;
     if (full) {
         c->pf_full_iters += 1;
         c->pf_since_full = 0;
-        conv = rn <= c->pf_target;
+        conv = rr <= target2;
         // FP32: a confirming evaluation that improved little on the previous explicit
         // residual has reached the rounding level of Jv - b
-        if (!conv && sizeof(T) == 4 && c->pf_confirm && rn >= 0.5 * c->pf_last_full) conv = true;
-        c->pf_last_full = rn;
-        if (rn < c->pf_best) { c->pf_best = rn; c->pf_best_it = c->pf_it; }
+        if (!conv && sizeof(T) == 4 && c->pf_confirm && rr >= 0.25 * c->pf_last_full) conv = true;
+        c->pf_last_full = rr;
+        if (rr < c->pf_best) { c->pf_best = rr; c->pf_best_it = c->pf_it; }
     } else {
         c->pf_since_full += 1;
-        if (rn <= c->pf_target) c->pf_force = 1;   // confirm with an explicit residual first
+        if (rr <= target2) c->pf_force = 1;   // confirm with an explicit residual first
     }
     // FP32 safety net: no new smallest explicit residual for PF_STALL iterations
     bool stalled = sizeof(T) == 4 && c->pf_it - c->pf_best_it >= PF_STALL;
@@ -756,7 +760,7 @@ struct FPfB1 {
         // a recurrence residual that meets the tolerance is confirmed by the explicit
         // J v - b of this same iteration, so that the solve stops at the iteration at
         // which Algorithm 1's explicit residual first meets it
-        const bool rec_conv = sqrt(tot[1]) <= c->pf_target;
+        const bool rec_conv = tot[1] <= c->pf_target * c->pf_target;
         const bool full = clamped || rec_conv || c->pf_force || c->pf_since_full + 1 >= PF_REFRESH;
         c->pf_full = full;
         c->pf_confirm = rec_conv || c->pf_force;
@@ -767,6 +771,79 @@ struct FPfB1 {
         }
     }
 };
+
+// One pixel of the fused iterate: J p = a p - kappa lap p, x = max(v + alpha p, v_con), the
+// recurrence residual R' = R + alpha J p, the flags (bit0 at the bound, bit1 active) and r' = R'
+// zeroed on the active set; acc[0..7]: clamped values, r'.r', r'.r, active values, and the sums
+// of the next direction (a r'^2, a r' p, a p^2, r' p over the free pixels).
+template <typename T>
+__device__ __forceinline__ uint8_t pf_iterate_px(T kappa, T alpha, double alpha_d, T p, T a, T v, T vc, T R0, T ro, T lp,
+                                                 T& x, T& R, T& rn, Acc<T>* acc) {
+    const T Jp = a * p - kappa * lp;
+    x = v + alpha * p;
+    if (x < vc) { x = vc; acc[0].count(T(1)); }
+    const bool at = (x == vc);
+    rn = R0 + alpha * Jp;
+    R = rn;
+    bool pos = false;
+    if (at) {   // the sign only matters at the bound (FP64 where FP32 is not decisive, as FPfB1)
+        if constexpr (sizeof(T) == 8) {
+            pos = rn > T(0);
+        } else {
+            T mag = fabs(R0) + fabs(alpha * Jp);
+            if (fabs(rn) > T(4e-7) * mag) pos = rn > T(0);
+            else pos = recur_positive_fp64(R0, alpha_d, Jp);
+        }
+    }
+    const bool active = at && pos;
+    if (active) rn = T(0);
+    acc[1].addp(rn, rn);
+    acc[2].addp(rn, ro);
+    if (active) acc[3].count(T(1));
+    if (!active) {   // sums of the next direction (free pixels)
+        const T ar = a * rn;
+        acc[4].addp(ar, rn);
+        acc[5].addp(ar, p);
+        acc[6].addp(a * p, p);
+        acc[7].addp(rn, p);
+    }
+    return (uint8_t)((at ? 1 : 0) | (active ? 2 : 0));
+}
+
+// One pixel of the explicit residual R = J x - b (lx = lap x) of a pixel at (or off) its bound:
+// flags and masked r' as above; acc[0..6]: r'.r', r'.r, active values, the sums of the next direction.
+template <typename T>
+__device__ __forceinline__ uint8_t pf_explicit_px(T kappa, double kd, T ro, T x, T a, T b, T p, bool at, T lx, T& R, T& rn,
+                                                  Acc<T>* acc) {
+    const T kl = kappa * lx;
+    rn = a * x - kl - b;
+    R = rn;
+    bool pos = false;
+    if (at) {   // the sign only matters at the bound
+        if constexpr (sizeof(T) == 8) {
+            pos = rn > T(0);
+        } else {
+            // FP32 residual; decide its sign in FP64 from the same FP32 operands when it
+            // is within rounding of zero (otherwise the FP32 sign is already exact)
+            T mag = fabs(a * x) + fabs(kl) + fabs(b);
+            if (fabs(rn) > T(4e-7) * mag) pos = rn > T(0);
+            else pos = resid_positive_fp64(a, x, kd, lx, b);
+        }
+    }
+    const bool active = at && pos;
+    if (active) rn = T(0);
+    acc[0].addp(rn, rn);
+    acc[1].addp(rn, ro);
+    if (active) acc[2].count(T(1));
+    if (!active) {   // sums of the next direction (free pixels; used by the three-pass iteration)
+        const T ar = a * rn;
+        acc[3].addp(ar, rn);
+        acc[4].addp(ar, p);
+        acc[5].addp(a * p, p);
+        acc[6].addp(rn, p);
+    }
+    return (uint8_t)((at ? 1 : 0) | (active ? 2 : 0));
+}
 
 template <typename T>
 struct FPfA3B {   // J p from the column pass's lap p, then the iterate of FPfB1
@@ -783,37 +860,11 @@ struct FPfA3B {   // J p from the column pass's lap p, then the iterate of FPfB1
         return In{d.th[2][i], d.r[0][i], d.th[0][i], d.r[2][i], d.lap[i], c.ro[i]};
     }
     __device__ static void pixel(const Desc<T>& d, const Ctx& c, size_t i, const In& a, T (&lp)[1], Acc<T>* acc) {
-        const T Jp = a.a * a.p - c.kappa * lp[0];
-        T x = a.v + c.alpha * a.p;
-        if (x < a.vc) { x = a.vc; acc[0].count(T(1)); }
+        T x, R, rn;
+        d.flags[i] = pf_iterate_px(c.kappa, c.alpha, c.alpha_d, a.p, a.a, a.v, a.vc, a.R, a.ro, lp[0], x, R, rn, acc);
         d.th[0][i] = x;
-        const bool at = (x == a.vc);
-        T rn = a.R + c.alpha * Jp;
-        d.lap[i] = rn;
-        bool pos = false;
-        if (at) {   // the sign only matters at the bound (FP64 where FP32 is not decisive, as FPfB1)
-            if constexpr (sizeof(T) == 8) {
-                pos = rn > T(0);
-            } else {
-                T mag = fabs(a.R) + fabs(c.alpha * Jp);
-                if (fabs(rn) > T(4e-7) * mag) pos = rn > T(0);
-                else pos = recur_positive_fp64(a.R, c.alpha_d, Jp);
-            }
-        }
-        const bool active = at && pos;
-        if (active) rn = T(0);
+        d.lap[i] = R;
         c.rn[i] = rn;
-        d.flags[i] = (uint8_t)((at ? 1 : 0) | (active ? 2 : 0));
-        acc[1].addp(rn, rn);
-        acc[2].addp(rn, a.ro);
-        if (active) acc[3].count(T(1));
-        if (!active) {   // sums of the next direction (free pixels)
-            const T ar = a.a * rn;
-            acc[4].addp(ar, rn);
-            acc[5].addp(ar, a.p);
-            acc[6].addp(a.a * a.p, a.p);
-            acc[7].addp(rn, a.p);
-        }
     }
     __device__ static void finalize(const Desc<T>& d, const double* tot) {
         FPfB1<T>::finalize(d, tot);
@@ -854,36 +905,10 @@ struct FPfB3 {   // explicit R = J v - b, active set {bound and R > 0}, beta, co
         return In{c.ro[i], d.th[0][i], d.r[0][i], d.r[1][i], d.th[2][i], d.flags[i]};
     }
     __device__ static void pixel(const Desc<T>& d, const Ctx& c, size_t i, const In& in, T (&v)[1], Acc<T>* acc) {
-        const T ro = in.ro, x = in.x, a = in.a, b = in.b, kl = c.kappa * v[0];
-        T rn = a * x - kl - b;
-        d.lap[i] = rn;
-        const bool at = in.fl & 1;
-        bool pos = false;
-        if (at) {   // the sign only matters at the bound
-            if constexpr (sizeof(T) == 8) {
-                pos = rn > T(0);
-            } else {
-                // FP32 residual; decide its sign in FP64 from the same FP32 operands when it
-                // is within rounding of zero (otherwise the FP32 sign is already exact)
-                T mag = fabs(a * x) + fabs(kl) + fabs(b);
-                if (fabs(rn) > T(4e-7) * mag) pos = rn > T(0);
-                else pos = resid_positive_fp64(a, x, c.kd, v[0], b);
-            }
-        }
-        const bool active = at && pos;
-        if (active) rn = T(0);
+        T R, rn;
+        d.flags[i] = pf_explicit_px(c.kappa, c.kd, in.ro, in.x, in.a, in.b, in.p, (in.fl & 1) != 0, v[0], R, rn, acc);
+        d.lap[i] = R;
         c.rn[i] = rn;   // beside the previous residual (kept for the preconditioned beta)
-        d.flags[i] = (uint8_t)((at ? 1 : 0) | (active ? 2 : 0));
-        acc[0].addp(rn, rn);
-        acc[1].addp(rn, ro);
-        if (active) acc[2].count(T(1));
-        if (!active) {   // sums of the next direction (free pixels; used by the three-pass iteration)
-            const T ar = a * rn;
-            acc[3].addp(ar, rn);
-            acc[4].addp(ar, in.p);
-            acc[5].addp(a * in.p, in.p);
-            acc[6].addp(rn, in.p);
-        }
     }
     __device__ static void finalize(const Desc<T>& d, const double* tot) {
         d.ctrl->pf_rsel ^= 1;
