@@ -233,6 +233,9 @@ static size_t problem_bytes(int nx, int ny, int prec) {
     return b;
 }
 
+// sizes whose solves run cluster-resident (k_resident.cu)
+static bool resident_size(int nx, int ny) { return nx <= 256 && ny <= 256 && nx * ny <= RESIDENT_PIXELS; }
+
 static bool valid_n(int n) { return n >= 16 && n <= 2048 && (n & (n - 1)) == 0; }
 
 // CUDA graphs of the two fixed launch sequences of a load step (a chunk of CG
@@ -482,6 +485,25 @@ static bool mech_cluster_group(const Group& g) {
         return false;
     }
 }
+// A sub-problem solve of a group of small FP32 grids in one launch, a cluster per problem
+// (k_resident.cu; kind 0 mechanics, 1 phase field).  The per-kernel path stays for other sizes,
+// FP64, the preconditioned and the four-pass BCCG and kernel timing (which times its kernels), and
+// where the device cannot host the cluster: false, nothing launched.
+template <typename T>
+static bool resident_solve(int kind, const Group& g) {
+    if constexpr (sizeof(T) == 4) {
+        if (!resident_size(g.nx, g.ny) || timing_on() || (kind == 1 && (g.precond || g_bccg4.load()))) return false;
+        const Desc<float>* d = (const Desc<float>*)g.d_desc;
+        cudaError_t e = kind == 0 ? launch_resident_mech(d, g.nx, g.ny, g.np, g.st)
+                                  : launch_resident_bccg(d, g.nx, g.ny, g.np, g.st);
+        if (e != cudaSuccess) cudaGetLastError();
+        return e == cudaSuccess;
+    } else {
+        (void)kind;
+        (void)g;
+        return false;
+    }
+}
 static int g_persist_share = 8;    // the persistent launch takes 1/share of the resident capacity
 
 template <typename T>
@@ -701,6 +723,7 @@ static int mech_solve_group(Group& g, int max_cg, int max_newton, pff_problem* e
     const int nx = g.nx, ny = g.ny, wp = g.wp, np = g.np;
     cudaStream_t st = g.st;
     int rc;
+    if (resident_solve<T>(0, g)) return 0;   // folds the last update itself
     if (mech_cluster_group<T>(g)) return 0;
     for (int round = 0; round <= max_newton; ++round) {
         launch_row_fwd<T>(RF_NEWTON, nx, ny, d, np, st);
@@ -750,10 +773,12 @@ static int pf_solve_group(Group& g, int max_pf, pff_problem* eh, bool& warmed) {
             cudaGetLastError();   // not launched (e.g. not enough resident capacity): chunked path
         }
     }
-    for (int it = 0; it <= max_pf + CHUNK; it += CHUNK) {
-        run_chunk<T>(1, g, warmed);
-        if ((rc = poll<T>(g, false, eh))) return rc;
-        if (all_bits(g, 4)) break;
+    if (!resident_solve<T>(1, g)) {
+        for (int it = 0; it <= max_pf + CHUNK; it += CHUNK) {
+            run_chunk<T>(1, g, warmed);
+            if ((rc = poll<T>(g, false, eh))) return rc;
+            if (all_bits(g, 4)) break;
+        }
     }
     launch_elem<T>(EL_POST, g.nx, g.ny, d, g.np, g.st);
     return 0;
@@ -1390,7 +1415,7 @@ int pff_solve_mechanics(pff_problem* h, pff_step_report* out) {
         using T = decltype(tag);
         const Desc<T>* d = (const Desc<T>*)h->d_desc;
         launch_step_begin<T>(d, 1, h->st);
-        if (mech_cluster_group<T>(g)) return poll<T>(g, true, h);
+        if (resident_solve<T>(0, g) || mech_cluster_group<T>(g)) return poll<T>(g, true, h);
         for (int round = 0; round <= p.mech_max_newton; ++round) {
             run_trio<T>(h, RF_NEWTON, CO_GAMMA_N, RI_NEWTON);
             for (int it = 0; it <= p.mech_max_cg + CHUNK; it += CHUNK) {
@@ -1438,6 +1463,7 @@ int pff_solve_phase_field(pff_problem* h, pff_step_report* out) {
                 cudaGetLastError();
             }
         }
+        if (resident_solve<T>(1, g)) return poll<T>(g, true, h);
         for (int it = 0; it <= p.pf_max_iter + CHUNK; it += CHUNK) {
             for (int c = 0; c < CHUNK; ++c) {
                 if (p.pf_precondition || g_bccg4.load()) {

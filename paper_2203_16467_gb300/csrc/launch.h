@@ -25,6 +25,11 @@ template <typename T> void launch_pf_cond(const Desc<T>* d, int np, cudaGraphCon
 // the whole mechanics solve of np FP32 512 x 512 problems, one thread-block cluster each (k_cluster.cu)
 bool mech_cluster_supported();
 cudaError_t launch_mech_cluster(const Desc<float>* d, int np, cudaStream_t st);
+// the solves of np small FP32 problems, one cluster each (k_resident.cu), for sizes up to 256 per side
+// and RESIDENT_PIXELS; cudaErrorNotSupported (nothing launched) otherwise
+constexpr int RESIDENT_PIXELS = 1 << 14;
+cudaError_t launch_resident_mech(const Desc<float>* d, int nx, int ny, int np, cudaStream_t st);
+cudaError_t launch_resident_bccg(const Desc<float>* d, int nx, int ny, int np, cudaStream_t st);
 void launch_convert_d2f(float* dst, const double* src, size_t n, cudaStream_t st);
 void launch_convert_f2d(double* dst, const float* src, size_t n, cudaStream_t st);
 
