@@ -231,6 +231,39 @@ __device__ __forceinline__ DF df_add(DF a, DF b) {
     float h = s + e;
     return DF{h, e - (h - s)};
 }
+// Double-float arithmetic on values (relative error a few 2^-46 away from cancellation and from the
+// ends of the exponent range): exact sum and product of floats, product, scaling, square root.
+__device__ __forceinline__ DF df_sum(float a, float b) {
+    float s = a + b, z = s - a;
+    return DF{s, (a - (s - z)) + (b - z)};
+}
+__device__ __forceinline__ DF df_of(double x) {
+    float h = (float)x;
+    return DF{h, (float)(x - (double)h)};
+}
+__device__ __forceinline__ DF df_neg(DF a) { return DF{-a.hi, -a.lo}; }
+__device__ __forceinline__ DF df_scale(DF a, float s) { return DF{a.hi * s, a.lo * s}; }   // s a power of two
+__device__ __forceinline__ DF df_mul(DF a, DF b) {
+    float p = __fmul_rn(a.hi, b.hi);
+    float e = fmaf(a.hi, b.hi, -p) + fmaf(a.hi, b.lo, a.lo * b.hi);
+    float h = p + e;
+    return DF{h, e - (h - p)};
+}
+__device__ __forceinline__ DF df_mulf(DF a, float b) {
+    float p = __fmul_rn(a.hi, b);
+    float e = fmaf(a.hi, b, -p) + a.lo * b;
+    float h = p + e;
+    return DF{h, e - (h - p)};
+}
+// one Newton step on the FP32 root (a.hi > 0)
+__device__ __forceinline__ DF df_sqrt(DF a) {
+    float r = rsqrtf(a.hi), x = a.hi * r;
+    float p = __fmul_rn(x, x);
+    float rem = ((a.hi - p) - fmaf(x, x, -p)) + a.lo;   // a - x^2 (a.hi - p is exact)
+    float e = 0.5f * r * rem;
+    float h = x + e;
+    return DF{h, e - (h - x)};
+}
 
 template <typename V> struct RedOps;
 template <> struct RedOps<double> {
@@ -421,6 +454,43 @@ __device__ __forceinline__ T psi_voldev(T xx, T yy, T xy, T lam, T mu) {
     T tr = xx + yy, K = lam + T(2) * mu / T(3), t3 = tr / T(3);
     T a = xx - t3, b = yy - t3, trp = rp(tr);
     return T(0.5) * K * trp * trp + mu * (a * a + b * b + T(2) * xy * xy);
+}
+
+// psi_0^+ of the crack-driving-force model in double-float arithmetic, for FP32 problems (GB300 runs
+// FP64 at 1/64 of the FP32 rate).  `small`: the operands are too near the ends of the FP32 exponent
+// range for the low parts (the caller then takes the FP64 function).
+struct DF3 { DF xx, yy, xy; };
+__device__ __forceinline__ DF df_pos(DF a) { return a.hi > 0.f ? a : DF{0.f, 0.f}; }
+__device__ __forceinline__ bool df_psi_range(const DF3& e, float lam, float mu) {
+    const float m = fmaxf(fmaxf(fabsf(e.xx.hi), fabsf(e.yy.hi)), fabsf(e.xy.hi));
+    const float k = fmaxf(fabsf(lam), mu);
+    return m > 1e-10f && m < 1e10f && k > 1e-15f && k < 1e15f;
+}
+__device__ __forceinline__ DF df_psi_plus(int split, const DF3& e, DF lam, DF mu) {
+    const int s = driving_of(split);
+    const DF tr = df_add(e.xx, e.yy);
+    if (s == ISOTROPIC) {
+        DF q = df_add(df_mul(e.xx, e.xx), df_mul(e.yy, e.yy));
+        q = df_add(q, df_scale(df_mul(e.xy, e.xy), 2.f));
+        return df_add(df_mul(df_scale(lam, 0.5f), df_mul(tr, tr)), df_mul(mu, q));
+    }
+    const DF trp = df_pos(tr);
+    if (s == VOLDEV) {
+        // a^2 + b^2 + 2 xy^2 with a = xx - tr/3, b = yy - tr/3 is xx^2 + yy^2 + 2 xy^2 - 4/9 tr^2
+        const DF tr2 = df_mul(tr, tr);
+        const DF third{0.33333334f, -9.934108e-09f}, k49{0.44444445f, -3.3113692e-09f};   // 1/3, 4/9
+        DF q = df_add(df_mul(e.xx, e.xx), df_mul(e.yy, e.yy));
+        q = df_add(q, df_scale(df_mul(e.xy, e.xy), 2.f));
+        q = df_add(q, df_neg(df_mul(k49, tr2)));
+        const DF K = df_add(lam, df_scale(df_mul(mu, third), 2.f));
+        return df_add(df_mul(df_scale(K, 0.5f), df_mul(trp, trp)), df_mul(mu, q));
+    }
+    const DF d = df_scale(df_add(e.xx, df_neg(e.yy)), 0.5f);
+    const DF s2 = df_add(df_mul(d, d), df_mul(e.xy, e.xy));
+    const DF rad = s2.hi > 0.f ? df_sqrt(s2) : DF{0.f, 0.f};
+    const DF h = df_scale(tr, 0.5f);
+    const DF a1 = df_pos(df_add(h, rad)), a2 = df_pos(df_add(h, df_neg(rad)));
+    return df_add(df_mul(df_scale(lam, 0.5f), df_mul(trp, trp)), df_mul(mu, df_add(df_mul(a1, a1), df_mul(a2, a2))));
 }
 
 // psi_0^+ of the crack-driving-force model.

@@ -5,7 +5,7 @@ namespace pff {
 
 template <typename T, class F>
 static void go_elem(int nx, int ny, const Desc<T>* d, int np, cudaStream_t st) {
-    launch_pdl<T>(k_elem<T, F>, dim3(elem_blocks(nx, ny, np), np), dim3(EL_NT), 0, st, d);
+    launch_pdl<T>(k_elem<T, F>, dim3(elem_blocks(nx, ny), np), dim3(EL_NT), 0, st, d);
     count_launch();
 }
 
@@ -18,7 +18,7 @@ void launch_elem(int op, int nx, int ny, const Desc<T>* d, int np, cudaStream_t 
         case EL_PF_INIT: go_elem<T, FPfInit<T>>(nx, ny, d, np, st); break;
         case EL_POST: go_elem<T, FPost<T>>(nx, ny, d, np, st); break;
         case EL_DF:
-            k_df<T><<<dim3(elem_blocks(nx, ny, np), np), EL_NT, 0, st>>>(d);
+            k_df<T><<<dim3(elem_blocks(nx, ny), np), EL_NT, 0, st>>>(d);
             count_launch();
             break;
         case EL_CONSTITUTIVE: go_elem<T, FConstitutive<T>>(nx, ny, d, np, st); break;

@@ -19,7 +19,8 @@
 //   column pass (FFT along y, mode multiplier, inverse) stores its rows straight into the row owners'.
 // What bounds it: the chain of dependent exchanges and scalars of an iteration (7300 cycles of a 64^2
 // CG iteration, of which the two spectrum exchanges take 1900 and the sums' 1500; at 128^2 the bytes
-// of the exchanges too: scattered remote stores move about 6 B per cycle and SM).  Measured on the chip: a cluster barrier with stores before it 960 (8 CTAs) to 1480 (16) cycles, a store with
+// of the exchanges too: scattered remote stores move about 6 B per cycle and SM).  Measured on the
+// chip: a cluster barrier with stores before it 960 (8 CTAs) to 1480 (16) cycles, a store with
 // transaction count (st.async) seen by the receiver after 240; an FP64 add 65, a division 550, a
 // square root 600 cycles.  Hence
 //   * every exchange is st.async with the bytes counted by an mbarrier of the receiver;

@@ -72,22 +72,79 @@ __global__ void k_gather(const Desc<T>* __restrict__ descs, int np, int* out) {
 // -F_phi = D + R_f with D = 2(1-phi) psi_0^+ and R_f = -c (f'(phi) - 2 ell^2 lap phi),
 // evaluated in FP64; first maximiser in row-major order; max D; then the
 // rescale decision of Algorithm 4 lines 4-10 (readings in the oracle docs).
+//
+// Only pixels that can hold one of the two maxima are evaluated in FP64: each value is first bounded
+// in FP32 (value and error bound), the block takes the largest lower bound, and a pixel whose upper
+// bound is below it is done.  The FP64 pipe runs at 1/64 of the FP32 rate; with every pixel in FP64
+// and one thread merging the blocks' results this kernel took 96 us at 512^2, 886 us at 2048^2
+// (eight 512^2 problems 280 us).
 struct ArgMax {
-    double v, D, R, Dmax;
-    long long i;
+    long long k;              // order-preserving integer image of the value (no FP64 comparisons)
+    double D, R;
+    long long i, Dk;          // index; image of the largest D
 };
+constexpr long long AM_NONE = (long long)0x8000000000000000ull;   // below every number
+// integer image of a double: the order of the integers is the order of the numbers; NaN below all
+__device__ __forceinline__ long long am_key(double x) {
+    if (x != x) return AM_NONE;
+    const long long b = __double_as_longlong(x + 0.0);
+    return b ^ ((b >> 63) & 0x7fffffffffffffffll);
+}
+__device__ __forceinline__ double am_value(long long k) {
+    return k == AM_NONE ? -INFINITY : __longlong_as_double(k ^ ((k >> 63) & 0x7fffffffffffffffll));
+}
 __device__ __forceinline__ void am_merge(ArgMax& a, const ArgMax& b) {
-    if (b.v > a.v || (b.v == a.v && b.i < a.i)) { a.v = b.v; a.i = b.i; a.D = b.D; a.R = b.R; }
-    a.Dmax = fmax(a.Dmax, b.Dmax);
+    if (b.k > a.k || (b.k == a.k && b.i < a.i)) { a.k = b.k; a.i = b.i; a.D = b.D; a.R = b.R; }
+    if (b.Dk > a.Dk) a.Dk = b.Dk;
 }
 __device__ __forceinline__ ArgMax am_shfl(const ArgMax& a, int o) {
     ArgMax b;
-    b.v = __shfl_down_sync(0xffffffffu, a.v, o);
+    b.k = __shfl_down_sync(0xffffffffu, a.k, o);
     b.D = __shfl_down_sync(0xffffffffu, a.D, o);
     b.R = __shfl_down_sync(0xffffffffu, a.R, o);
-    b.Dmax = __shfl_down_sync(0xffffffffu, a.Dmax, o);
+    b.Dk = __shfl_down_sync(0xffffffffu, a.Dk, o);
     b.i = __shfl_down_sync(0xffffffffu, a.i, o);
     return b;
+}
+// block total in thread 0
+__device__ __forceinline__ ArgMax am_block(ArgMax best, ArgMax (&sh)[EL_NT / 32]) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) am_merge(best, am_shfl(best, o));
+    if (lane == 0) sh[warp] = best;
+    __syncthreads();
+    if (threadIdx.x == 0)
+        for (int w = 1; w < EL_NT / 32; ++w) am_merge(best, sh[w]);
+    return best;
+}
+// integer image of a float, as am_key
+__device__ __forceinline__ int am_keyf(float x) {
+    const int b = __float_as_int(x);
+    return x != x ? (int)0x80000000 : b ^ ((b >> 31) & 0x7fffffff);
+}
+
+// FP32 values of -F_phi and D of one pixel with bounds of their errors.  With M the largest of
+// |eps_bar| + |eps*| over the components, FP32 strains are off by 2e-7 M, eigenvalues by 1e-6 M and
+// psi_0^+ by less than (2 |lambda| + 12 mu) 1e-6 M^2, rounding of the inputs of an FP64 problem included;
+// the bound taken is (16 |lambda| + 32 mu) 1e-6 M^2, 4e-6 of the other terms, and 1e-30 for the end of
+// the exponent range.  An overflow gives a NaN or infinite bound: the pixel is then evaluated in FP64.
+struct DfBound { float v, dv, D, dD; };
+template <typename T>
+__device__ __forceinline__ DfBound df_bound(const Desc<T>& d, const Consts& k, const float (&eb)[3], float lc, float mc, float c,
+                                            float kap, unsigned i) {
+    const float e0 = (float)d.eps[0][i], e1 = (float)d.eps[1][i], e2 = (float)d.eps[2][i];
+    const float E = (float)d.E[i], ph = (float)d.phi[i], lap = (float)d.lap[i];
+    const float lam = lc * E, mu = mc * E;
+    const float psi = psi_plus<float>(k.split, eb[0] + e0, eb[1] + e1, eb[2] + e2, lam, mu);
+    const float M = fmaxf(fmaxf(fabsf(eb[0]) + fabsf(e0), fabsf(eb[1]) + fabsf(e1)), fabsf(eb[2]) + fabsf(e2));
+    const float g = 2.f * (1.f - ph);
+    const float cf = k.fracture == AT1 ? c : 2.f * c * ph, kl = kap * lap;
+    DfBound r;
+    r.D = g * psi;
+    r.dD = (2.f + 2.f * fabsf(ph)) * (16e-6f * fabsf(lam) + 32e-6f * mu) * M * M + 4e-6f * fabsf(r.D) + 1e-30f;
+    r.v = r.D - cf + kl;
+    r.dv = r.dD + 4e-6f * (fabsf(cf) + fabsf(kl));
+    return r;
 }
 
 template <typename T>
@@ -95,57 +152,90 @@ __global__ void __launch_bounds__(EL_NT) k_df(const Desc<T>* __restrict__ descs)
     const Desc<T>& d = descs[blockIdx.y];
     const Consts& k = d.k;
     Ctrl* ctrl = d.ctrl;
-    double eb[3];
-    for (int j = 0; j < 3; ++j) eb[j] = ldd(&ctrl->eps_bar[j]);
-    ArgMax best{-INFINITY, 0.0, 0.0, -INFINITY, 0x7fffffffffffffffLL};
-    const size_t n = (size_t)d.nx * d.ny;
-    for (size_t i = (size_t)blockIdx.x * EL_NT + threadIdx.x; i < n; i += (size_t)gridDim.x * EL_NT) {
-        double E = (double)d.E[i];
-        double psi = psi_plus<double>(k.split, eb[0] + (double)d.eps[0][i], eb[1] + (double)d.eps[1][i],
-                                      eb[2] + (double)d.eps[2][i], k.lam_c * E, k.mu_c * E);
-        double ph = (double)d.phi[i];
-        double D = 2.0 * (1.0 - ph) * psi;
-        double fp = k.fracture == AT1 ? 1.0 : 2.0 * ph;
-        double R = -k.c * fp + k.kappa * (double)d.lap[i];
-        double v = D + R;
-        if (v > best.v) { best.v = v; best.i = (long long)i; best.D = D; best.R = R; }
-        best.Dmax = fmax(best.Dmax, D);
-    }
+    constexpr int U = 8;               // pixels of a thread per round
     __shared__ ArgMax sh[EL_NT / 32];
+    __shared__ int lov[EL_NT / 32], loD[EL_NT / 32];
     __shared__ int s_last;
+    double eb[3];
+    float ebf[3];
+    for (int j = 0; j < 3; ++j) { eb[j] = ldd(&ctrl->eps_bar[j]); ebf[j] = (float)eb[j]; }
+    const float lc = (float)k.lam_c, mc = (float)k.mu_c, cf = (float)k.c, kap = (float)k.kappa;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    for (int o = 16; o > 0; o >>= 1) { ArgMax b = am_shfl(best, o); am_merge(best, b); }
-    if (lane == 0) sh[warp] = best;
-    __syncthreads();
+    ArgMax best{AM_NONE, 0.0, 0.0, 0x7fffffffffffffffLL, AM_NONE};
+    const unsigned n = (unsigned)d.nx * d.ny, stride = gridDim.x * EL_NT;
+    int bv = (int)0x80000000, bD = bv;   // largest lower bounds of the block so far
+    for (unsigned base = blockIdx.x * EL_NT + threadIdx.x; base - threadIdx.x < n; base += U * stride) {
+        float uv[U], uD[U];            // upper bounds
+#pragma unroll
+        for (int u = 0; u < U; ++u) {
+            const unsigned i = base + u * stride;
+            if (i < n) {
+                const DfBound r = df_bound(d, k, ebf, lc, mc, cf, kap, i);
+                uv[u] = r.v + r.dv;
+                uD[u] = r.D + r.dD;
+                bv = max(bv, am_keyf(r.v - r.dv));
+                bD = max(bD, am_keyf(r.D - r.dD));
+            }
+        }
+        bv = __reduce_max_sync(0xffffffffu, bv);
+        bD = __reduce_max_sync(0xffffffffu, bD);
+        __syncthreads();               // the previous round's bounds have been read
+        if (lane == 0) { lov[warp] = bv; loD[warp] = bD; }
+        __syncthreads();
+#pragma unroll
+        for (int w = 0; w < EL_NT / 32; ++w) { bv = max(bv, lov[w]); bD = max(bD, loD[w]); }
+#pragma unroll 1
+        for (int u = 0; u < U; ++u) {
+            const unsigned i = base + u * stride;
+            if (i >= n) break;
+            float xv = uv[0], xD = uD[0];
+#pragma unroll
+            for (int q = 1; q < U; ++q)
+                if (q == u) { xv = uv[q]; xD = uD[q]; }
+            // (a NaN bound compares as below every number: not decided in FP32)
+            if (xv == xv && xD == xD && am_keyf(xv) < bv && am_keyf(xD) < bD) continue;
+            double E = (double)d.E[i];
+            double psi = psi_plus<double>(k.split, eb[0] + (double)d.eps[0][i], eb[1] + (double)d.eps[1][i],
+                                          eb[2] + (double)d.eps[2][i], k.lam_c * E, k.mu_c * E);
+            double ph = (double)d.phi[i];
+            double D = 2.0 * (1.0 - ph) * psi;
+            double fp = k.fracture == AT1 ? 1.0 : 2.0 * ph;
+            double R = -k.c * fp + k.kappa * (double)d.lap[i];
+            const ArgMax m{am_key(D + R), D, R, (long long)i, am_key(D)};
+            am_merge(best, m);
+        }
+    }
+    best = am_block(best, sh);
     double* part = d.part;
     if (threadIdx.x == 0) {
-        ArgMax a = sh[0];
-        for (int w = 1; w < EL_NT / 32; ++w) am_merge(a, sh[w]);
         size_t o = (size_t)blockIdx.x * 5;
-        __stcg(&part[o + 0], a.v); __stcg(&part[o + 1], a.D); __stcg(&part[o + 2], a.R);
-        __stcg(&part[o + 3], a.Dmax); __stcg(&part[o + 4], (double)a.i);
+        __stcg(&part[o + 0], __longlong_as_double(best.k)); __stcg(&part[o + 1], best.D); __stcg(&part[o + 2], best.R);
+        __stcg(&part[o + 3], __longlong_as_double(best.Dk)); __stcg(&part[o + 4], __longlong_as_double(best.i));
         __threadfence();
         unsigned t = atomicAdd(&ctrl->counter, 1u);
         s_last = (t == gridDim.x - 1);
     }
     __syncthreads();
-    if (!s_last || threadIdx.x != 0) return;
+    if (!s_last) return;
     __threadfence();
-    ArgMax a{-INFINITY, 0.0, 0.0, -INFINITY, 0x7fffffffffffffffLL};
-    for (unsigned b = 0; b < gridDim.x; ++b) {
-        ArgMax c{__ldcg(&part[b * 5 + 0]), __ldcg(&part[b * 5 + 1]), __ldcg(&part[b * 5 + 2]),
-                 __ldcg(&part[b * 5 + 3]), (long long)__ldcg(&part[b * 5 + 4])};
+    ArgMax a{AM_NONE, 0.0, 0.0, 0x7fffffffffffffffLL, AM_NONE};
+    for (unsigned b = threadIdx.x; b < gridDim.x; b += EL_NT) {
+        const ArgMax c{__double_as_longlong(__ldcg(&part[b * 5 + 0])), __ldcg(&part[b * 5 + 1]), __ldcg(&part[b * 5 + 2]),
+                       __double_as_longlong(__ldcg(&part[b * 5 + 4])), __double_as_longlong(__ldcg(&part[b * 5 + 3]))};
         am_merge(a, c);
     }
+    a = am_block(a, sh);
+    if (threadIdx.x != 0) return;
+    const double av = am_value(a.k), aD = am_value(a.Dk);
     ctrl->counter = 0u;
-    ctrl->mF_max = a.v;
-    ctrl->D_max = a.Dmax;
+    ctrl->mF_max = av;
+    ctrl->D_max = aD;
     ctrl->istar = (int)a.i;
     ctrl->Rf_star = a.R;
     ctrl->D_star = a.D;
-    if (a.v > k.Fmax && a.Dmax > k.thresh) ctrl->flag = 1;
+    if (av > k.Fmax && aD > k.thresh) ctrl->flag = 1;
     double g = 1.0;
-    if (a.v > k.Fmax && ctrl->flag) {
+    if (av > k.Fmax && ctrl->flag) {
         double num = k.Fmax - a.R, den = a.D;
         if (num > 0.0 && den > 0.0) {
             g = sqrt(num / den);
@@ -337,14 +427,15 @@ void go_col(const Desc<T>* d, int np, int nm, cudaStream_t st, int key) {
         default: break;                             \
     }
 
-inline int elem_blocks(int nx, int ny, int np) {
-    long long n = (long long)nx * ny;
-    long long b = (n + EL_NT * 4 - 1) / (EL_NT * 4);
-    long long cap = 2048;
-    if (b > cap) b = cap;
-    if (b < 1) b = 1;
-    (void)np;
-    return (int)b;
+// Up to 256^2 one pixel per thread, so that a small grid's few pixels spread over the SMs (64^2: the
+// BCCG start 24 -> 13 us, post-step 16 -> 14 us; 256^2: 26 -> 13 us); four per thread, whose loads
+// are in flight together, beyond (one per thread at 512^2: post-step of one simulation 18 -> 23 us, of
+// eight 46 -> 75 us, for the reductions of four times the blocks).  The number of problems does not
+// enter: the summation order, and with it every bit, is the same in every launch group.
+inline int elem_blocks(int nx, int ny) {
+    const long long n = (long long)nx * ny, one = (n + EL_NT - 1) / EL_NT;
+    const long long b = one <= 256 ? one : (n + EL_NT * 4 - 1) / (EL_NT * 4);
+    return (int)(b > 2048 ? 2048 : b < 1 ? 1 : b);
 }
 
 }  // namespace pff

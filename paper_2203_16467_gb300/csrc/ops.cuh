@@ -393,10 +393,21 @@ struct FCopyOut {
 // BCCG start (Algorithm 1 lines 1-5) after the rescale of lines 4-10 of Algorithm 4:
 // eps <- gamma eps; a = eta/dt + 2 psi_0^+ + c f''; b = -F_phi(phi_n);
 // v_con = phi_con(phi_n) - phi_n <= 0; v^0 = 0; r^0 = -b masked; p^0 = -r^0.
+//
+// psi_0^+, a and b are formed in FP64 and stored in the problem's precision.  FP32 problems form them
+// in double-float arithmetic instead (the same FP32 values but for one in some 2^20; FP64 only near
+// the ends of the FP32 exponent range): the FP64 pipe bound this kernel (one 512^2 problem 39 -> 19 us,
+// eight 213 -> 77 us, 2048^2 410 -> 142 us; now the issue of some 400 instructions per pixel).
+static __device__ __noinline__ double psi_plus_fp64(int split, double xx, double yy, double xy, double lam, double mu) {
+    return psi_plus<double>(split, xx, yy, xy, lam, mu);
+}
 template <typename T>
 struct FPfInit {
     static constexpr int NR = 4;
-    struct Ctx { double g; int resc; double eb[3]; double eta_dt; int frozen; };
+    struct Ctx {
+        double g; int resc; double eb[3]; double eta_dt; int frozen;
+        DF ebf[3], lc, mc, ac, cf, kap;   // double-float: eps_bar, lambda/E, mu/E, eta/dt + c f'', c (AT1) or 2 c (AT2), kappa
+    };
     __device__ static bool skip(const Desc<T>&) { return false; }
     __device__ static Ctx prep(const Desc<T>& d) {
         Ctx c;
@@ -405,6 +416,14 @@ struct FPfInit {
         for (int k = 0; k < 3; ++k) c.eb[k] = c.g * ldd(&d.ctrl->eps_bar[k]);
         c.eta_dt = ldflag(&d.ctrl->use_override) ? ldd(&d.ctrl->eta_dt_override) : d.k.eta_dt;
         c.frozen = ldflag(&d.ctrl->con_frozen);
+        if constexpr (sizeof(T) == 4) {
+            for (int k = 0; k < 3; ++k) c.ebf[k] = df_of(c.eb[k]);
+            c.lc = df_of(d.k.lam_c);
+            c.mc = df_of(d.k.mu_c);
+            c.ac = df_of(c.eta_dt + d.k.cf2);
+            c.cf = df_of(d.k.fracture == AT1 ? d.k.c : 2.0 * d.k.c);
+            c.kap = df_of(d.k.kappa);
+        }
         return c;
     }
     __device__ static void pixel(const Desc<T>& d, const Ctx& c, size_t i, Acc<T>* acc) {
@@ -415,14 +434,33 @@ struct FPfInit {
             e0 *= g; e1 *= g; e2 *= g;
             d.eps[0][i] = e0; d.eps[1][i] = e1; d.eps[2][i] = e2;
         }
-        double E = (double)d.E[i];
-        double lam = k.lam_c * E, mu = k.mu_c * E;
-        double psi = psi_plus<double>(k.split, c.eb[0] + (double)e0, c.eb[1] + (double)e1, c.eb[2] + (double)e2, lam, mu);
         T ph = d.phi[i];
-        double phd = (double)ph;
-        double fp = k.fracture == AT1 ? 1.0 : 2.0 * phd;
-        T a = T(c.eta_dt + 2.0 * psi + k.cf2);
-        T b = T(2.0 * (1.0 - phd) * psi - k.c * fp + k.kappa * (double)d.lap[i]);
+        T a, b;
+        if constexpr (sizeof(T) == 4) {
+            const float E = d.E[i], lap = d.lap[i];
+            const DF3 e{df_add(c.ebf[0], DF{e0, 0.f}), df_add(c.ebf[1], DF{e1, 0.f}), df_add(c.ebf[2], DF{e2, 0.f})};
+            const DF lam = df_mulf(c.lc, E), mu = df_mulf(c.mc, E);
+            DF psi2;
+            if (df_psi_range(e, lam.hi, mu.hi))
+                psi2 = df_scale(df_psi_plus(k.split, e, lam, mu), 2.f);
+            else
+                psi2 = df_of(2.0 * psi_plus_fp64(k.split, c.eb[0] + (double)e0, c.eb[1] + (double)e1, c.eb[2] + (double)e2,
+                                                 k.lam_c * (double)E, k.mu_c * (double)E));
+            const DF av = df_add(c.ac, psi2);
+            DF bv = df_mul(df_sum(1.f, -ph), psi2);
+            bv = df_add(bv, df_neg(k.fracture == AT1 ? c.cf : df_mulf(c.cf, ph)));
+            bv = df_add(bv, df_mulf(c.kap, lap));
+            a = av.hi + av.lo;
+            b = bv.hi + bv.lo;
+        } else {
+            double E = (double)d.E[i];
+            double lam = k.lam_c * E, mu = k.mu_c * E;
+            double psi = psi_plus<double>(k.split, c.eb[0] + (double)e0, c.eb[1] + (double)e1, c.eb[2] + (double)e2, lam, mu);
+            double phd = (double)ph;
+            double fp = k.fracture == AT1 ? 1.0 : 2.0 * phd;
+            a = T(c.eta_dt + 2.0 * psi + k.cf2);
+            b = T(2.0 * (1.0 - phd) * psi - k.c * fp + k.kappa * (double)d.lap[i]);
+        }
         T pcon = c.frozen ? d.aux[i] : ((k.irrev == CRACK_SET) ? (ph >= T(k.crack_thr) ? ph : T(0)) : ph);
         T vcon = pcon - ph;
         T v = T(0) < vcon ? vcon : T(0);
