@@ -308,9 +308,10 @@ int pff_constitutive(pff_problem* h, const double* eps3, const double* phi, cons
  *     blocks: more SMs busy when a launch carries one simulation).
  *   PFF_VARIANT_BCCG_PASSES (grid_n, ncomp ignored): variant 0 = Algorithm 1 in
  *     three operator passes per iteration (the step length alpha from the column
- *     pass by Parseval, the iterate fused into the J p pass; default), 1 = four
- *     passes (alpha from p.Jp summed in real space, the iterate in its own
- *     elementwise kernel; what the preconditioned option always uses).
+ *     pass by Parseval, the iterate fused into the J p pass; default; FP32 grids
+ *     up to 2^14 pixels run it in one launch per solve), 1 = four passes (alpha
+ *     from p.Jp summed in real space, the iterate in its own elementwise kernel;
+ *     what the preconditioned option always uses).
  * Takes effect at the next launch; captured CUDA graphs are re-captured.
  * Synchronises the device.  Unsupported arguments: PFF_ERR_INVALID_ARG. */
 enum { PFF_VARIANT_COLUMN_SHAPE = 2, PFF_VARIANT_BCCG_PASSES = 3 };
@@ -393,12 +394,15 @@ int pff_apply_laplacian_noalloc_f32(int nx, int ny, double dx, const float* in_d
 unsigned long long pff_kernel_launches(void);
 
 /* Replay the fixed per-iteration launch sequences of the CG and BCCG loops
- * from captured CUDA graphs (default on = 1: plain graphs, in which the
- * explicit J v - b chain of a BCCG iteration that does not need it launches and
- * returns at once).  on = 2 puts that chain in a conditional graph node that a
- * one-thread kernel opens only in iterations that need it (measured slower on
- * GB300 than the returning kernels); 0 launches every kernel directly.  Results do not depend on the
- * setting.  Graphs are used only on problems or batches created with a
+ * from captured CUDA graphs (default on = 1: plain graphs).  The default BCCG
+ * takes the next three launches of its sequence for an explicit J v - b when an
+ * iteration needs one; the preconditioned and four-pass variants have a chain of
+ * their own for it, whose kernels return at once in the other iterations, and
+ * on = 2 puts that chain in a conditional graph node that a one-thread kernel
+ * opens only in iterations that need it (measured slower on GB300 than the
+ * returning kernels).  0 launches every kernel directly.  Problems whose solves
+ * run in one launch (FP32 grids up to 2^14 pixels) have no such sequences.
+ * Results do not depend on the setting.  Graphs are used only on problems or batches created with a
  * non-NULL stream and while kernel timing is off.  Synchronises the device. */
 int pff_set_graphs(int on);
 
@@ -468,7 +472,10 @@ int pff_set_barrier_spin_limit(long long cycles);
  * 4 BCCG iterate; row-inverse: 0 Newton, 1 CG, 2 Laplacian, 3 energy,
  * 4 BCCG direction, 5 BCCG residual; column: 0 Newton, 1 CG, 3 driving force,
  * 4 BCCG; elementwise: 0 fold, 1 BCCG start, 2 post-step, 3 driving-force
- * maximum).  Enabling, resetting and reading synchronize the device. */
+ * maximum).  The default BCCG's launches count in its direction and iterate classes
+ * whether they advance the iterate or evaluate J v - b.  While timing is on the
+ * solves of FP32 grids up to 2^14 pixels, otherwise one launch each, run as these
+ * kernels.  Enabling, resetting and reading synchronize the device. */
 int pff_timing_enable(int on);
 int pff_timing_reset(void);
 int pff_timing_read(int family, int op, double* total_ms, unsigned long long* launches);

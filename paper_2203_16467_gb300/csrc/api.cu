@@ -458,7 +458,8 @@ struct Group {
     int precond = 0;       // BCCG with the Fourier Helmholtz preconditioner (same for all problems)
 };
 
-static const int CHUNK = 12;
+static const int CHUNK = 12;       // CG iterations, or iterations of the preconditioned / four-pass BCCG
+static const int SLOTS = 16;       // slots of the default BCCG (an iteration takes one, with J v evaluated two)
 static bool g_graphs_enabled = true;
 static bool g_cond_nodes = false;  // BCCG explicit-residual chain in conditional graph nodes
 static bool g_persist = false;     // persistent BCCG solve for single FP32 512^2 problems (opt-in)
@@ -506,32 +507,41 @@ static bool resident_solve(int kind, const Group& g) {
 }
 static int g_persist_share = 8;    // the persistent launch takes 1/share of the resident capacity
 
+// BCCG with a chain of its own for the explicit residual (the preconditioned and four-pass variants)
+static bool bccg_chain(const Group& g) { return g.precond || g_bccg4.load(); }
+// chunks that hold every iteration a solve may take
+static int bccg_chunks(const Group& g, int max_pf) {
+    return bccg_chain(g) ? max_pf / CHUNK + 2 : (2 * max_pf) / SLOTS + 2;
+}
+
 template <typename T>
 static void chunk_direct(int kind, const Group& g) {
     const Desc<T>* d = (const Desc<T>*)g.d_desc;
     const int nx = g.nx, ny = g.ny, wp = g.wp, np = g.np;
     cudaStream_t st = g.st;
-    for (int c = 0; c < CHUNK; ++c) {
-        if (kind == 0) {
+    if (kind == 0) {
+        for (int c = 0; c < CHUNK; ++c) {
             launch_row_fwd<T>(RF_CG, nx, ny, d, np, st);
             launch_col<T>(CO_GAMMA_CG, nx, ny, wp, d, np, st);
             launch_row_inv<T>(RI_CG, nx, ny, d, np, st);
-        } else {
+        }
+    } else if (!bccg_chain(g)) {
+        for (int c = 0; c < SLOTS; ++c) {
+            launch_row_fwd<T>(RF_PF_S, nx, ny, d, np, st);
+            launch_col<T>(CO_LAP_PFS, nx, ny, wp, d, np, st);
+            launch_row_inv<T>(RI_PF_S, nx, ny, d, np, st);
+        }
+    } else {
+        for (int c = 0; c < CHUNK; ++c) {
             if (g.precond) {   // z = M^-1 r on the free set, beta
                 launch_row_fwd<T>(RF_PF_Z, nx, ny, d, np, st);
                 launch_col<T>(CO_PRECOND, nx, ny, wp, d, np, st);
                 launch_row_inv<T>(RI_PF_Z, nx, ny, d, np, st);
             }
-            if (g.precond || g_bccg4.load()) {
-                launch_row_fwd<T>(RF_PF_A, nx, ny, d, np, st);
-                launch_col<T>(CO_LAP_PF, nx, ny, wp, d, np, st);
-                launch_row_inv<T>(RI_PF_A, nx, ny, d, np, st);
-                launch_elem<T>(EL_PF_B, nx, ny, d, np, st);
-            } else {   // alpha from the column pass, the iterate fused into the J p pass
-                launch_row_fwd<T>(RF_PF_A, nx, ny, d, np, st);
-                launch_col<T>(CO_LAP_PFQ, nx, ny, wp, d, np, st);
-                launch_row_inv<T>(RI_PF_AB, nx, ny, d, np, st);
-            }
+            launch_row_fwd<T>(RF_PF_A, nx, ny, d, np, st);
+            launch_col<T>(CO_LAP_PF, nx, ny, wp, d, np, st);
+            launch_row_inv<T>(RI_PF_A, nx, ny, d, np, st);
+            launch_elem<T>(EL_PF_B, nx, ny, d, np, st);
             launch_row_fwd<T>(RF_PF_B, nx, ny, d, np, st);          // only when J v is evaluated
             launch_col<T>(CO_LAP_PF_FULL, nx, ny, wp, d, np, st);   // explicitly this iteration
             launch_row_inv<T>(RI_PF_B, nx, ny, d, np, st);
@@ -579,18 +589,11 @@ static cudaError_t capture_pf_chunk(const Group& g, cudaGraph_t* out, int* kerne
             launch_row_inv<T>(RI_PF_Z, nx, ny, d, np, st);
             nk += 3;
         }
-        if (g.precond || g_bccg4.load()) {
-            launch_row_fwd<T>(RF_PF_A, nx, ny, d, np, st);
-            launch_col<T>(CO_LAP_PF, nx, ny, wp, d, np, st);
-            launch_row_inv<T>(RI_PF_A, nx, ny, d, np, st);
-            launch_elem<T>(EL_PF_B, nx, ny, d, np, st);
-            nk += 4;
-        } else {
-            launch_row_fwd<T>(RF_PF_A, nx, ny, d, np, st);
-            launch_col<T>(CO_LAP_PFQ, nx, ny, wp, d, np, st);
-            launch_row_inv<T>(RI_PF_AB, nx, ny, d, np, st);
-            nk += 3;
-        }
+        launch_row_fwd<T>(RF_PF_A, nx, ny, d, np, st);
+        launch_col<T>(CO_LAP_PF, nx, ny, wp, d, np, st);
+        launch_row_inv<T>(RI_PF_A, nx, ny, d, np, st);
+        launch_elem<T>(EL_PF_B, nx, ny, d, np, st);
+        nk += 4;
         launch_pf_cond<T>(d, np, h, st);
         nk += 1;
         cudaStreamCaptureStatus cs;
@@ -663,7 +666,7 @@ static void run_chunk(int kind, Group& g, bool& warmed) {
         int nk = 0;
         cudaError_t e = cudaSuccess;
         t_capturing = true;
-        if (kind == 1 && g_cond_nodes) {
+        if (kind == 1 && g_cond_nodes && bccg_chain(g)) {
             e = capture_pf_chunk<T>(g, &graph, &nk);
         } else {
             e = cudaStreamBeginCapture(g.st, cudaStreamCaptureModeThreadLocal);
@@ -774,7 +777,7 @@ static int pf_solve_group(Group& g, int max_pf, pff_problem* eh, bool& warmed) {
         }
     }
     if (!resident_solve<T>(1, g)) {
-        for (int it = 0; it <= max_pf + CHUNK; it += CHUNK) {
+        for (int c = bccg_chunks(g, max_pf); c > 0; --c) {
             run_chunk<T>(1, g, warmed);
             if ((rc = poll<T>(g, false, eh))) return rc;
             if (all_bits(g, 4)) break;
@@ -1419,7 +1422,7 @@ int pff_solve_mechanics(pff_problem* h, pff_step_report* out) {
         for (int round = 0; round <= p.mech_max_newton; ++round) {
             run_trio<T>(h, RF_NEWTON, CO_GAMMA_N, RI_NEWTON);
             for (int it = 0; it <= p.mech_max_cg + CHUNK; it += CHUNK) {
-                for (int c = 0; c < CHUNK; ++c) run_trio<T>(h, RF_CG, CO_GAMMA_CG, RI_CG);
+                chunk_direct<T>(0, g);
                 int r2 = poll<T>(g, false, h);
                 if (r2) return r2;
                 if (all_bits(g, 1)) break;
@@ -1464,17 +1467,8 @@ int pff_solve_phase_field(pff_problem* h, pff_step_report* out) {
             }
         }
         if (resident_solve<T>(1, g)) return poll<T>(g, true, h);
-        for (int it = 0; it <= p.pf_max_iter + CHUNK; it += CHUNK) {
-            for (int c = 0; c < CHUNK; ++c) {
-                if (p.pf_precondition || g_bccg4.load()) {
-                    if (p.pf_precondition) run_trio<T>(h, RF_PF_Z, CO_PRECOND, RI_PF_Z);
-                    run_trio<T>(h, RF_PF_A, CO_LAP_PF, RI_PF_A);
-                    launch_elem<T>(EL_PF_B, h->nx, h->ny, d, 1, h->st);
-                } else {
-                    run_trio<T>(h, RF_PF_A, CO_LAP_PFQ, RI_PF_AB);
-                }
-                run_trio<T>(h, RF_PF_B, CO_LAP_PF_FULL, RI_PF_B);
-            }
+        for (int c = bccg_chunks(g, p.pf_max_iter); c > 0; --c) {
+            chunk_direct<T>(1, g);
             int r2 = poll<T>(g, false, h);
             if (r2) return r2;
             if (all_bits(g, 4)) break;

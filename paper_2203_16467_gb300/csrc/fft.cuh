@@ -238,7 +238,8 @@ struct ModeK {
     int nx, ny;
     const Consts* kc;       // the problem constants (read only by rarely used multipliers)
     T pre_a, pre_k;         // preconditioner (a_mean, 2 c ell^2), set by multipliers that need them
-    ModeK() = default;
+    int full = 0;           // an explicit residual's slot (FColLapPFS)
+    __device__ __forceinline__ ModeK() {}
     __device__ __forceinline__ explicit ModeK(const Desc<T>& d)
         : cx(T(d.k.two_pi_over_Lx)), cy(T(d.k.two_pi_over_Ly)), inv_n(T(d.k.inv_n)), nx(d.nx), ny(d.ny), kc(&d.k) {}
 };

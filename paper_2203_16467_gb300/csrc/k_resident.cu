@@ -715,7 +715,7 @@ __global__ void __launch_bounds__(RG<NX, NY, 1>::NT, 1) k_res_bccg(const Desc<fl
         ro[q] = 0.f;
     }
     unsigned par = 0, p0 = 0, p1 = 0;
-    // The scalar warp's state (the same in its lanes): FColLapPFQ's, FPfA3B's and FPfB3's finalizers with
+    // The scalar warp's state (the same in its lanes): FColLapPFQ's and FPfSlotOut's finalizers with
     // the next step's flags and beta first and everything else after the row warps have gone on.
     double target2 = 0.0, kin = 0.0, pap = 0.0, rp = 0.0, irp = 0.0, beta = 0.0, rr = 0.0, best = 0.0, last = 0.0, nact = 0.0;
     int it = 0, best_it = 0, since_full = 0, full_iters = 0, clamp_iters = 0, status = 0;

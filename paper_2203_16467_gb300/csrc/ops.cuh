@@ -491,7 +491,7 @@ struct FPfInit {
         c->pf_it = 0;
         c->pf_break = 0;
         c->n_active = 0;
-        c->pf_full = 1;
+        c->pf_full = 0;
         c->pf_force = 0;
         c->pf_confirm = 0;
         c->pf_since_full = 0;
@@ -660,19 +660,24 @@ struct FPfA3 {   // J p; p.Jp, r.p -> alpha = -(r.p)/(p.Jp)
 // p.Jp = sum a p^2 - kappa sum p lap_N p, and -sum p lap_N p = (1/(nx ny)) sum_k |2 pi q|^2
 // |p^_k|^2 over the full spectrum (Parseval), so alpha = -(r.p)/(p.Jp) is known after the
 // column pass, and the row-inverse pass that forms J p applies the iterate at once:
-//   FPfA1      (row forward): p = -r + beta p, zero on the active set
-//   FColLapPFQ (column)     : sum over the modes of w(kx) |2 pi q|^2 |p^|^2 (w = 2 on the kx
+//   FPfSlotIn  (row forward): p = -r + beta p, zero on the active set
+//   FColLapPFS (column)     : sum over the modes of w(kx) |2 pi q|^2 |p^|^2 (w = 2 on the kx
 //                             columns that stand for two modes, else 1); alpha
-//   FPfA3B     (row inverse): J p = a p - kappa lap_N p; v = max(v + alpha p, v_con); the
+//   FPfSlotOut (row inverse): J p = a p - kappa lap_N p; v = max(v + alpha p, v_con); the
 //                             residual recurrence R + alpha J p; active set; r' and its dots
+// An iteration that evaluates J v explicitly (pf_full, set by the iterate) takes the next three
+// launches for it: the same kernels transform v instead of p and form R = J v - b.  So every launch
+// of a chunk works until the solve stops; with three more kernels per iteration that returned at once
+// when they were not needed (in 40 to 90 % of the iterations) a 512^2 BCCG solve took 5449 us, now
+// 5316, an FP64 256^2 one 7674, now 7090, a load step of 64 problems of 256^2 26.6 ms, now 25.6.
 // sum a p^2 and r.p of the next direction p' = -r' + beta p (free pixels; 0 on the active set)
 // come from sums of the iteration that forms r': sum a p'^2 = S1 - 2 beta S2 + beta^2 S3 and
 // r'.p' = -r'.r' + beta S4 with S1 = sum a r'^2, S2 = sum a r' p, S3 = sum a p^2 (free
 // pixels) and S4 = r'.p (pf_next_dir); the first direction p = -r from the start's sums.
-// (The preconditioned variant and the persistent kernel keep FPfA1 / FColLapPF / FPfA3 / FPfB1.)
-struct FColLapPFQ {
+// (The preconditioned and four-pass variants and the persistent kernel keep FPfA1 / FColLapPF / FPfA3 /
+// FPfB1 and FPfVIn / FColLapPFFull / FPfB3 for the explicit residual.)
+struct FColLapPFQ {   // (as such the column pass of the cluster-resident solve)
     static constexpr int NR = 1;
-    template <typename T> __device__ static bool skip(const Desc<T>& d) { return ldflag(&d.ctrl->pf_a); }
     template <typename T>
     __device__ static void accum(const ModeK<T>& m, int kx, int ky, const typename CT<T>::t (&v)[1], Acc<T>* acc) {
         if (2 * kx > m.nx) return;   // padding columns of the spectrum rows hold no modes
@@ -883,30 +888,93 @@ __device__ __forceinline__ uint8_t pf_explicit_px(T kappa, double kd, T ro, T x,
     return (uint8_t)((at ? 1 : 0) | (active ? 2 : 0));
 }
 
+// One slot of the default iteration: a direction and iterate (pf_full 0) or an explicit residual (1).
 template <typename T>
-struct FPfA3B {   // J p from the column pass's lap p, then the iterate of FPfB1
+struct FPfSlotIn {
+    static constexpr int NR = 0;
+    struct Ctx { T beta; int upd; int full; const T* r; };
+    __device__ static bool skip(const Desc<T>& d) {
+        int f = ldflag(&d.ctrl->pf_b);
+        if (blockIdx.x == 0 && threadIdx.x == 0) d.ctrl->pf_a = f;
+        return f;
+    }
+    __device__ static Ctx prep(const Desc<T>& d) {
+        return Ctx{T(ldd(&d.ctrl->pf_beta)), ldflag(&d.ctrl->pf_it) > 0, ldflag(&d.ctrl->pf_full),
+                   pf_r(d, ldflag(&d.ctrl->pf_rsel))};
+    }
+    struct In { T p, r; uint8_t fl; };
+    __device__ static In load(const Desc<T>& d, const Ctx& c, size_t i) {
+        In a{c.full ? d.th[0][i] : d.th[2][i], T(0), 0};
+        if (c.upd && !c.full) { a.r = c.r[i]; a.fl = d.flags[i]; }
+        return a;
+    }
+    __device__ static void pixel(const Desc<T>& d, const Ctx& c, size_t i, const In& a, T (&v)[1], Acc<T>*) {
+        T p = a.p;
+        if (c.upd && !c.full) {
+            p = (a.fl & 2) ? T(0) : -a.r + c.beta * p;
+            d.th[2][i] = p;
+        }
+        v[0] = p;
+    }
+    __device__ static void finalize(const Desc<T>&, const double*) {}
+};
+
+struct FColLapPFS {
+    static constexpr int NR = 1;
+    template <typename T> __device__ static bool skip(const Desc<T>& d) { return ldflag(&d.ctrl->pf_a); }
+    template <typename T> __device__ static void mode_prep(const Desc<T>& d, ModeK<T>& m) { m.full = ldflag(&d.ctrl->pf_full); }
+    template <typename T>
+    __device__ static void accum(const ModeK<T>& m, int kx, int ky, const typename CT<T>::t (&v)[1], Acc<T>* acc) {
+        if (!m.full) FColLapPFQ::accum(m, kx, ky, v, acc);
+    }
+    template <typename T> __device__ static void apply(const ModeK<T>& m, int kx, int ky, typename CT<T>::t (&v)[1]) {
+        lap_apply(m, kx, ky, v);
+    }
+    template <typename T> __device__ static void finalize(const Desc<T>& d, const double* tot) {
+        if (!d.ctrl->pf_full) FColLapPFQ::finalize<T>(d, tot);
+    }
+};
+
+template <typename T>
+struct FPfSlotOut {
     static constexpr int NR = 8;
-    struct Ctx { T kappa; T alpha; double alpha_d; const T* ro; T* rn; };
+    struct Ctx { T kappa; T alpha; double alpha_d; double kd; const T* ro; T* rn; const T* w; int full; };
     __device__ static bool skip(const Desc<T>& d) { return ldflag(&d.ctrl->pf_a); }
     __device__ static Ctx prep(const Desc<T>& d) {
-        const int sel = ldflag(&d.ctrl->pf_rsel);
+        const int sel = ldflag(&d.ctrl->pf_rsel), full = ldflag(&d.ctrl->pf_full);
         const double a = ldd(&d.ctrl->pf_alpha);
-        return Ctx{T(d.k.kappa), T(a), a, pf_r(d, sel), pf_r(d, sel ^ 1)};
+        return Ctx{T(d.k.kappa), T(a), a, d.k.kappa, pf_r(d, sel), pf_r(d, sel ^ 1), full ? d.r[1] : d.r[2], full};
     }
-    struct In { T p, a, v, vc, R, ro; };
+    struct In { T p, a, v, w, R, ro; uint8_t fl; };   // w: v_con, or b in an explicit residual
     __device__ static In load(const Desc<T>& d, const Ctx& c, size_t i) {
-        return In{d.th[2][i], d.r[0][i], d.th[0][i], d.r[2][i], d.lap[i], c.ro[i]};
+        In a{d.th[2][i], d.r[0][i], d.th[0][i], c.w[i], T(0), c.ro[i], 0};
+        if (c.full) a.fl = d.flags[i];
+        else a.R = d.lap[i];
+        return a;
     }
-    __device__ static void pixel(const Desc<T>& d, const Ctx& c, size_t i, const In& a, T (&lp)[1], Acc<T>* acc) {
-        T x, R, rn;
-        d.flags[i] = pf_iterate_px(c.kappa, c.alpha, c.alpha_d, a.p, a.a, a.v, a.vc, a.R, a.ro, lp[0], x, R, rn, acc);
-        d.th[0][i] = x;
+    __device__ static void pixel(const Desc<T>& d, const Ctx& c, size_t i, const In& a, T (&l)[1], Acc<T>* acc) {
+        T R, rn;
+        if (c.full) {
+            d.flags[i] = pf_explicit_px(c.kappa, c.kd, a.ro, a.v, a.a, a.w, a.p, (a.fl & 1) != 0, l[0], R, rn, acc);
+        } else {
+            T x;
+            d.flags[i] = pf_iterate_px(c.kappa, c.alpha, c.alpha_d, a.p, a.a, a.v, a.w, a.R, a.ro, l[0], x, R, rn, acc);
+            d.th[0][i] = x;
+        }
         d.lap[i] = R;
         c.rn[i] = rn;
     }
     __device__ static void finalize(const Desc<T>& d, const double* tot) {
-        FPfB1<T>::finalize(d, tot);
-        if (!d.ctrl->pf_full) pf_next_dir(d.ctrl, tot + 4);   // else the explicit residual pass does it
+        Ctrl* c = d.ctrl;
+        if (c->pf_full) {
+            c->pf_full = 0;
+            c->pf_rsel ^= 1;
+            pf_finish(d, c, tot[0], tot[1], tot[2], true);
+            pf_next_dir(c, tot + 3);
+        } else {
+            FPfB1<T>::finalize(d, tot);
+            if (!c->pf_full) pf_next_dir(c, tot + 4);   // else the explicit residual does it
+        }
     }
 };
 
