@@ -390,8 +390,9 @@ static int upload_desc(pff_problem* h) {
 // when it is page-locked) and one kernel, with no conversion loop on the host.
 static bool ensure_stage(pff_problem* h) { return h->stage != nullptr; }
 
-// Copy nx*ny FP64 values (host or device) into a field of the problem's precision.
-static int put_field(pff_problem* h, void* dst, const double* src, size_t count, int on_device) {
+// Queue the copy of FP64 values (host or device) into a field of the problem's precision; the
+// source may be reused once the stream has been synchronised (put_field does so).
+static int queue_field(pff_problem* h, void* dst, const double* src, size_t count, int on_device) {
     cudaError_t e = cudaSuccess;
     if (h->prec == PFF_FP64) {
         e = cudaMemcpyAsync(dst, src, count * 8, on_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice, h->st);
@@ -410,7 +411,12 @@ static int put_field(pff_problem* h, void* dst, const double* src, size_t count,
         e = cudaMemcpyAsync(dst, tmp.data(), count * 4, cudaMemcpyHostToDevice, h->st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
     }
-    if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);   // the caller may reuse its buffer on return
+    return e == cudaSuccess ? 0 : cuda_fail(h, e, "copy in");
+}
+static int put_field(pff_problem* h, void* dst, const double* src, size_t count, int on_device) {
+    const int rc = queue_field(h, dst, src, count, on_device);
+    if (rc) return rc;
+    const cudaError_t e = cudaStreamSynchronize(h->st);   // the caller may reuse its buffer on return
     return e == cudaSuccess ? 0 : cuda_fail(h, e, "copy in");
 }
 
@@ -444,6 +450,14 @@ static int write_ctrl(pff_problem* h) {
     return e == cudaSuccess ? 0 : cuda_fail(h, e, "write control block");
 }
 
+// Write one member of the control block (its value already in the pinned mirror) and synchronise.
+static int write_member(pff_problem* h, const void* member, size_t bytes) {
+    const size_t off = (const char*)member - (const char*)h->h_ctrl;
+    cudaError_t e = cudaMemcpyAsync((char*)h->ctrl + off, member, bytes, cudaMemcpyHostToDevice, h->st);
+    if (e == cudaSuccess) e = cudaStreamSynchronize(h->st);
+    return e == cudaSuccess ? 0 : cuda_fail(h, e, "write control block");
+}
+
 // ---------------------------------------------------------------------------
 // A group: problems of equal (nx, ny, precision) whose kernels share launches.
 struct Group {
@@ -455,6 +469,7 @@ struct Group {
     int* h_flags;          // pinned np
     Ctrl* h_ctrl;          // pinned np
     GraphCache* graphs;    // may be null (no graphs)
+    Ctrl* one = nullptr;   // the control block of a group of one
     int precond = 0;       // BCCG with the Fourier Helmholtz preconditioner (same for all problems)
 };
 
@@ -703,6 +718,15 @@ static int poll(Group& g, bool ctrl_too, pff_problem* eh) {
     const Desc<T>* d = (const Desc<T>*)g.d_desc;
     cudaError_t e = take_launch_error();
     if (e != cudaSuccess) return cuda_fail(eh, e, "kernel launch");
+    if (g.one) {   // one copy of the control block itself
+        e = cudaMemcpyAsync(g.h_ctrl, g.one, sizeof(Ctrl), cudaMemcpyDeviceToHost, g.st);
+        if (e == cudaSuccess) e = cudaStreamSynchronize(g.st);
+        if (e != cudaSuccess) return cuda_fail(eh, e, "poll");
+        const Ctrl& c = g.h_ctrl[0];
+        g.h_flags[0] = (c.cg_b ? 1 : 0) | (c.nd_a ? 2 : 0) | (c.pf_b ? 4 : 0);
+        if (timing_on()) timing_collect();
+        return 0;
+    }
     launch_gather<T>(d, g.np, g.d_flags, ctrl_too ? (void*)g.d_ctrl : nullptr, g.st);
     e = cudaMemcpyAsync(g.h_flags, g.d_flags, sizeof(int) * g.np, cudaMemcpyDeviceToHost, g.st);
     if (e == cudaSuccess && ctrl_too)
@@ -843,6 +867,7 @@ static Group single_group(pff_problem* h) {
     g.h_flags = h->h_flags;
     g.h_ctrl = h->h_ctrl;
     g.graphs = &h->graphs;
+    g.one = h->ctrl;
     g.precond = h->prm.pf_precondition != 0;
     return g;
 }
@@ -1007,6 +1032,7 @@ struct BatchGroup {
     Ctrl* h_ctrl = nullptr;
     GraphCache* graphs = nullptr;
     cudaStream_t stream = nullptr;   // own stream: groups of different shapes overlap on the device
+    std::vector<Desc<double>> sent;  // what d_desc holds
 };
 
 }  // namespace pff
@@ -1063,6 +1089,7 @@ static int build_groups(pff_batch* b) {
                 old.cap >= (int)g.slots.size()) {
                 g.cap = old.cap; g.d_desc = old.d_desc; g.d_flags = old.d_flags; g.d_ctrl = old.d_ctrl;
                 g.h_flags = old.h_flags; g.h_ctrl = old.h_ctrl; g.graphs = old.graphs; g.stream = old.stream;
+                g.sent.swap(old.sent);
                 old.d_desc = nullptr; old.d_flags = nullptr; old.d_ctrl = nullptr; old.h_flags = nullptr; old.h_ctrl = nullptr;
                 old.graphs = nullptr; old.stream = nullptr;
                 break;
@@ -1090,14 +1117,19 @@ static int build_groups(pff_batch* b) {
     // descriptors (parameters may have changed since the last step)
     for (auto& g : b->groups) {
         std::vector<Desc<double>> hd(g.slots.size());
+        std::memset((void*)hd.data(), 0, sizeof(Desc<double>) * hd.size());
         for (size_t j = 0; j < g.slots.size(); ++j) {
             pff_problem* h = b->slot[g.slots[j]];
             if (g.prec == PFF_FP64) hd[j] = make_desc<double>(h);
             else { Desc<float> f = make_desc<float>(h); std::memcpy(&hd[j], &f, sizeof(f)); }
         }
+        // unchanged since the last upload (the whole content): nothing to send
+        if (g.sent.size() == hd.size() && !std::memcmp(g.sent.data(), hd.data(), sizeof(Desc<double>) * hd.size())) continue;
+        g.sent.clear();
         cudaError_t e = cudaMemcpyAsync(g.d_desc, hd.data(), sizeof(Desc<double>) * hd.size(), cudaMemcpyHostToDevice, b->st);
         if (e == cudaSuccess) e = cudaStreamSynchronize(b->st);
         if (e != cudaSuccess) { b->err = cudaGetErrorString(e); return PFF_ERR_CUDA; }
+        g.sent.swap(hd);
     }
     return PFF_OK;
 }
@@ -1350,27 +1382,27 @@ int pff_set_strain(pff_problem* h, const double* eps_star, const double eps_bar[
     const size_t n = h->n();
     const size_t es = h->prec == PFF_FP64 ? 8 : 4;
     int rc;
-    for (int j = 0; j < 3; ++j) {
-        if (eps_star) {
-            if ((rc = put_field(h, h->field[2 + j], eps_star + j * n, n, on_device))) return rc;
-        } else {
-            cudaError_t e = cudaMemsetAsync(h->field[2 + j], 0, n * es, h->st);
-            if (e != cudaSuccess) return cuda_fail(h, e, "memset");
-        }
+    // the three planes are adjacent (n es is a multiple of 256): one copy, conversion or memset;
+    // host values of an FP32 problem pass through its staging buffer plane by plane
+    if (!eps_star) {
+        cudaError_t e = cudaMemsetAsync(h->field[2], 0, 3 * n * es, h->st);
+        if (e != cudaSuccess) return cuda_fail(h, e, "memset");
+    } else if (on_device || h->prec == PFF_FP64) {
+        if ((rc = queue_field(h, h->field[2], eps_star, 3 * n, on_device))) return rc;
+    } else {
+        for (int j = 0; j < 3; ++j)
+            if ((rc = queue_field(h, h->field[2 + j], eps_star + j * n, n, 0))) return rc;
     }
-    if ((rc = read_ctrl(h))) return rc;
     for (int j = 0; j < 3; ++j) h->h_ctrl->eps_bar[j] = eps_bar[j];
     h->broken = false;
     h->td_dt = -1.0;
-    return write_ctrl(h);
+    return write_member(h, h->h_ctrl->eps_bar, sizeof(h->h_ctrl->eps_bar));   // synchronises: the caller's buffer is free
 }
 
 int pff_set_flag(pff_problem* h, int flag) {
     if (!h) return PFF_ERR_INVALID_ARG;
-    int rc = read_ctrl(h);
-    if (rc) return rc;
     h->h_ctrl->flag = flag ? 1 : 0;
-    return write_ctrl(h);
+    return write_member(h, &h->h_ctrl->flag, sizeof(int));
 }
 
 int pff_step_load(pff_problem* h, int n_steps, pff_step_report* out, int* steps_done) {
@@ -1445,6 +1477,14 @@ int pff_solve_phase_field(pff_problem* h, pff_step_report* out) {
     if (!h) return PFF_ERR_INVALID_ARG;
     Group g = single_group(h);
     const pff_params& p = h->prm;
+    // phi += v by the post-step kernel with its strain increment off; then the control block
+    auto finish = [&]() -> int {
+        cudaError_t e = cudaMemsetAsync(&h->ctrl->post_mode, 1, sizeof(int), h->st);   // any value but 0
+        elem(h, EL_POST);
+        if (e == cudaSuccess) e = cudaMemsetAsync(&h->ctrl->post_mode, 0, sizeof(int), h->st);
+        if (e != cudaSuccess) return cuda_fail(h, e, "phase-field update");
+        return h->prec == PFF_FP64 ? poll<double>(g, true, h) : poll<float>(g, true, h);
+    };
     // rescale disabled for a bare sub-problem: gamma = 1
     auto body = [&](auto tag) -> int {
         using T = decltype(tag);
@@ -1461,41 +1501,31 @@ int pff_solve_phase_field(pff_problem* h, pff_step_report* out) {
                     if (r2) return r2;
                     if (g.h_ctrl[0].status & 8)
                         return fail(h, PFF_ERR_BARRIER_TIMEOUT, "persistent phase-field solve: a grid barrier timed out");
-                    return 0;
+                    return finish();
                 }
                 cudaGetLastError();
             }
         }
-        if (resident_solve<T>(1, g)) return poll<T>(g, true, h);
-        for (int c = bccg_chunks(g, p.pf_max_iter); c > 0; --c) {
-            chunk_direct<T>(1, g);
-            int r2 = poll<T>(g, false, h);
-            if (r2) return r2;
-            if (all_bits(g, 4)) break;
+        if (!resident_solve<T>(1, g)) {
+            for (int c = bccg_chunks(g, p.pf_max_iter); c > 0; --c) {
+                chunk_direct<T>(1, g);
+                int r2 = poll<T>(g, false, h);
+                if (r2) return r2;
+                if (all_bits(g, 4)) break;
+            }
         }
-        // phi += v without touching eps_bar: only the update of FPost is wanted, so run
-        // it and restore eps_bar afterwards
-        return poll<T>(g, true, h);
+        return finish();
     };
     int rc = h->prec == PFF_FP64 ? body(double()) : body(float());
     if (rc) return rc;
-    Ctrl saved = g.h_ctrl[0];
-    elem(h, EL_POST);
-    if ((rc = sync(h, "phase-field update"))) return rc;
-    if ((rc = read_ctrl(h))) return rc;
-    for (int j = 0; j < 3; ++j) h->h_ctrl->eps_bar[j] = saved.eps_bar[j];
-    Ctrl post = *h->h_ctrl;
-    if ((rc = write_ctrl(h))) return rc;
+    const Ctrl& c = g.h_ctrl[0];
     if (out) {
         std::memset(out, 0, sizeof(*out));
-        fill_report(post, h->split, out);
-        out->bccg_iters = saved.pf_it;
-        out->pf_res = std::sqrt(saved.pf_rr);
-        out->n_active = saved.n_active;
+        fill_report(c, h->split, out);
         out->incremented = 0;
-        for (int j = 0; j < 3; ++j) out->eps_bar[j] = saved.eps_bar[j];
+        for (int j = 0; j < 3; ++j) out->eps_bar[j] = c.eps_bar[j];
     }
-    return saved.status ? PFF_ERR_NOT_CONVERGED : PFF_OK;
+    return c.status ? PFF_ERR_NOT_CONVERGED : PFF_OK;
 }
 
 int pff_get_fields(pff_problem* h, int which, double* host_out) {
@@ -1819,6 +1849,7 @@ int pff_batch_step(pff_batch* b, int n_steps, pff_step_report* reports, int* ste
             g.st = bg.stream ? bg.stream : b->st;
             g.d_desc = bg.d_desc; g.d_flags = bg.d_flags; g.d_ctrl = bg.d_ctrl;
             g.h_flags = bg.h_flags; g.h_ctrl = bg.h_ctrl; g.graphs = bg.graphs; g.precond = bg.precond;
+            if (g.np == 1) g.one = h0->ctrl;
             rcs[gi] = run_group_step(g, p, energies, h0);
         };
         if (ng == 1) {
