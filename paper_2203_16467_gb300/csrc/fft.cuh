@@ -736,6 +736,187 @@ __global__ void __launch_bounds__(64 * CW) k_col512(const Desc<T>* __restrict__ 
 }
 
 // ---------------------------------------------------------------------------
+// Column pass for ny = 1024 and 2048 (FP32) with sixteen values of every component in a thread's
+// registers: ny = 16 x 16 x R3 (R3 = 4 or 8), N1 = ny / 16 threads per column.
+//   stage 1: thread t holds rows t + N1 m (m < 16): DFT16 over m -> k1, twiddle W_ny^(t k1)
+//   stage 2: thread (k1, a), a < R3, holds t = a + R3 b (b < 16): DFT16 over b -> k2, twiddle W_N1^(a k2)
+//   stage 3: thread t holds the groups g = k1 + 16 k2 = t + N1 q (q < 16 / R3): DFT R3 over a -> k3,
+//            modes ky = g + 256 k3
+// The multiplier acts on the NC components of a mode, which one thread holds, and the inverse runs the
+// stages backwards with the same twiddles conjugated, so a column makes two exchanges through shared
+// memory each way instead of the eight to ten passes of the Stockham form.  Exchange layouts per
+// component and column (column stride XS): stage-1 value (k1, t) at (N1 + R3) k1 + t, stage-2 value
+// (a, g) at (256 + P2) a + g; with XS = 16 / CW (mod 16) a half-warp's 8-byte accesses touch 16
+// different bank pairs.  Four columns (one 32-byte sector per row and access): with two, and two
+// blocks per SM, the line accesses of the loads and stores lead (2048^2 three components 77-104 us).
+// One launch, us, Stockham pass -> here: three components 2048^2 107 -> 75, 1024^2 27 -> 18; one
+// component 2048^2 33 -> 22, with the BCCG's sum 42 -> 26 (two blocks per SM; 1024^2 18 -> 14).  What is
+// left is latency: 16 warps per SM (98 registers of data a thread, 200 KB of exchange buffers).
+template <typename C, bool INV>
+__device__ __forceinline__ void dft16(C* u) {   // X[k] ends at u[4 (k mod 4) + k / 4]
+    using T = decltype(u[0].x);
+    const T c1 = T(0.92387953251128675613), s1 = T(0.38268343236508977173), h = T(0.70710678118654752440);
+    const C w1{c1, INV ? s1 : -s1}, w2{h, INV ? h : -h}, w3{s1, INV ? c1 : -c1};
+#pragma unroll
+    for (int n = 0; n < 4; ++n) dft4<C, INV>(u[n], u[4 + n], u[8 + n], u[12 + n]);
+    u[5] = cmul(u[5], w1);
+    u[6] = cmul(u[6], w2);
+    u[7] = cmul(u[7], w3);
+    u[9] = cmul(u[9], w2);
+    u[10] = INV ? C{-u[10].y, u[10].x} : C{u[10].y, -u[10].x};
+    u[11] = cmul(u[11], C{-h, INV ? h : -h});
+    u[13] = cmul(u[13], w3);
+    u[14] = cmul(u[14], C{-h, INV ? h : -h});
+    u[15] = cmul(u[15], C{-c1, INV ? -s1 : s1});
+#pragma unroll
+    for (int k = 0; k < 4; ++k) dft4<C, INV>(u[4 * k], u[4 * k + 1], u[4 * k + 2], u[4 * k + 3]);
+}
+__host__ __device__ constexpr int at16(int k) { return 4 * (k & 3) + (k >> 2); }   // place of X[k] after dft16
+
+template <typename T, int NY, int NC, int CW>
+struct Col16Cfg {
+    static constexpr int N1 = NY / 16, R3 = NY / 256, NT = CW * N1;
+    static constexpr int P1 = N1 + R3;                       // pitch of a stage-1 row
+    static constexpr int P2 = 256 + (CW == 2 && R3 == 4 ? 2 : 1);
+    static constexpr int NEED = cmax(16 * P1, R3 * P2), OFF = 16 / CW;
+    static constexpr int XS = ((NEED - OFF + 15) / 16) * 16 + OFF;
+    static constexpr size_t SMEM = (size_t)NC * CW * XS * sizeof(typename CT<T>::t);
+};
+
+// u[c][at(r)] *= w^r for r = 1 .. 15 (w^1, w^2, w^4, w^8 from the table tw[r step], the others products)
+template <typename C, int NC, bool CONJ, bool PERM>
+__device__ __forceinline__ void twiddle16(C (&u)[NC][16], const C* tw, int step) {
+    C w[16];
+#pragma unroll
+    for (int r = 1; r < 16; r *= 2) {
+        const C x = __ldg(tw + r * step);
+        w[r] = CONJ ? C{x.x, -x.y} : x;
+    }
+#pragma unroll
+    for (int r = 1; r < 16; ++r) {
+        const int hi = r >= 8 ? 8 : r >= 4 ? 4 : r >= 2 ? 2 : 1;
+        if (r != hi) w[r] = cmul(w[hi], w[r - hi]);
+#pragma unroll
+        for (int c = 0; c < NC; ++c) {
+            C& x = u[c][PERM ? at16(r) : r];
+            x = cmul(x, w[r]);
+        }
+    }
+}
+
+template <typename T, int NY, int NC, class OP, int CW>
+__global__ void __launch_bounds__(CW * NY / 16, NC == 1 && NY == 2048 ? 2 : 1) k_col16(const Desc<T>* __restrict__ descs) {
+    using Cfg = Col16Cfg<T, NY, NC, CW>;
+    using C = typename CT<T>::t;
+    constexpr int N1 = Cfg::N1, R3 = Cfg::R3, P1 = Cfg::P1, P2 = Cfg::P2, CS = CW * Cfg::XS, Q = 16 / R3;
+    const Desc<T>& d = descs[blockIdx.y];
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    pdl_enter();
+    ModeK<T> mk;
+    if (block_prep<ColPrep<T, OP>>(d, mk)) return;
+    const int j = threadIdx.x % CW, t = threadIdx.x / CW;
+    const int kx = blockIdx.x * CW + j;
+    C* xb = reinterpret_cast<C*>(smem_raw) + j * Cfg::XS;
+    const unsigned plane = (unsigned)d.ny * d.wp;   // 32-bit indices: < 2^32 elements
+    C* S = d.S + ((unsigned)t * d.wp + kx);
+    const unsigned step = (unsigned)N1 * d.wp;
+    const C* tw = d.tw + NY;
+    const int k1 = t / R3, a = t % R3;              // stage-2 role
+    C u[NC][16];
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+#pragma unroll
+        for (int m = 0; m < 16; ++m) u[c][m] = S[c * plane + m * step];
+    // forward
+#pragma unroll
+    for (int c = 0; c < NC; ++c) dft16<C, false>(u[c]);
+    twiddle16<C, NC, false, true>(u, tw, t);
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+#pragma unroll
+        for (int k = 0; k < 16; ++k) xb[c * CS + P1 * k + t] = u[c][at16(k)];
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+#pragma unroll
+        for (int b = 0; b < 16; ++b) u[c][b] = xb[c * CS + P1 * k1 + a + R3 * b];
+        dft16<C, false>(u[c]);
+    }
+    twiddle16<C, NC, false, true>(u, tw, 16 * a);
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+#pragma unroll
+        for (int k = 0; k < 16; ++k) xb[c * CS + P2 * a + 16 * k + k1] = u[c][at16(k)];
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+#pragma unroll
+            for (int r = 0; r < R3; ++r) u[c][q * R3 + r] = xb[c * CS + P2 * r + t + N1 * q];
+            if constexpr (R3 == 4) dft4<C, false>(u[c][4 * q], u[c][4 * q + 1], u[c][4 * q + 2], u[c][4 * q + 3]);
+            else dft8<C, false>(*reinterpret_cast<C(*)[8]>(&u[c][8 * q]));
+        }
+    // modes
+    constexpr int NRA = ColNR<OP>::value > 0 ? ColNR<OP>::value : 1;
+    Acc<T> acc[NRA];
+#pragma unroll
+    for (int q = 0; q < Q; ++q)
+#pragma unroll
+        for (int r = 0; r < R3; ++r) {
+            const int ky = t + N1 * q + 256 * r;
+            C v[NC];
+#pragma unroll
+            for (int c = 0; c < NC; ++c) v[c] = u[c][q * R3 + r];
+            if constexpr (ColNR<OP>::value > 0) OP::accum(mk, kx, ky, v, acc);
+            OP::apply(mk, kx, ky, v);
+#pragma unroll
+            for (int c = 0; c < NC; ++c) u[c][q * R3 + r] = v[c];
+        }
+    // inverse
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+#pragma unroll
+        for (int q = 0; q < Q; ++q) {
+            if constexpr (R3 == 4) dft4<C, true>(u[c][4 * q], u[c][4 * q + 1], u[c][4 * q + 2], u[c][4 * q + 3]);
+            else dft8<C, true>(*reinterpret_cast<C(*)[8]>(&u[c][8 * q]));
+#pragma unroll
+            for (int r = 0; r < R3; ++r) xb[c * CS + P2 * r + t + N1 * q] = u[c][q * R3 + r];
+        }
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+#pragma unroll
+        for (int k = 0; k < 16; ++k) u[c][k] = xb[c * CS + P2 * a + 16 * k + k1];
+    twiddle16<C, NC, true, false>(u, tw, 16 * a);
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        dft16<C, true>(u[c]);
+#pragma unroll
+        for (int b = 0; b < 16; ++b) xb[c * CS + P1 * k1 + a + R3 * b] = u[c][at16(b)];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int c = 0; c < NC; ++c)
+#pragma unroll
+        for (int k = 0; k < 16; ++k) u[c][k] = xb[c * CS + P1 * k + t];
+    twiddle16<C, NC, true, false>(u, tw, t);
+#pragma unroll
+    for (int c = 0; c < NC; ++c) {
+        dft16<C, true>(u[c]);
+#pragma unroll
+        for (int m = 0; m < 16; ++m) S[c * plane + m * step] = u[c][at16(m)];
+    }
+    if constexpr (ColNR<OP>::value > 0) {
+        double tot[ColNR<OP>::value];
+        if (reduce_acc<ColNR<OP>::value, Cfg::NT>(acc, d.part, &d.ctrl->counter, gridDim.x, tot) && threadIdx.x == 0)
+            OP::finalize(d, tot);
+    }
+}
+
+// ---------------------------------------------------------------------------
 // mode multipliers
 // Signed wavenumber index of row ky (numpy fftfreq order); Nyquist flagged.
 __device__ __forceinline__ int signed_k(int k, int n) { return k < n / 2 ? k : k - n; }

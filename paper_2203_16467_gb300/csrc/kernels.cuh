@@ -404,6 +404,12 @@ void go_col(const Desc<T>* d, int np, int nm, cudaStream_t st, int key) {
             smem_optin((const void*)fn, Cfg::SMEM);
             launch_pdl<T>(fn, dim3((nm + COL512_CW - 1) / COL512_CW, np), dim3(Cfg::NT), Cfg::SMEM, st, d);
         }
+    } else if constexpr (NY >= 1024 && sizeof(T) == 4) {   // register-resident radix-16 stages
+        constexpr int CW = 4;
+        using Cfg = Col16Cfg<T, NY, NC, CW>;
+        auto fn = k_col16<T, NY, NC, OP, CW>;
+        smem_optin((const void*)fn, Cfg::SMEM);
+        launch_pdl<T>(fn, dim3((nm + CW - 1) / CW, np), dim3(Cfg::NT), Cfg::SMEM, st, d);
     } else {
         using Cfg = ColCfg<T, NY, NC>;
         auto fn = k_col<T, NY, NC, OP>;
