@@ -191,19 +191,33 @@ struct RowCfg {
     // rows per block: about 512 complex values per block so that a 512^2 grid
     // already gives 128+ blocks per component plane
     static constexpr int ROWS = pow2floor(cmax(1, cmin(16, 512 / (NC * M))));   // divides every ny >= 16
-    static constexpr int NT = (NC * ROWS * M >= 1024) ? 256 : 128;
+    static constexpr bool F32 = sizeof(T) == 4;
+    // 128 threads for up to 1024 complex values (and the 1536 of an FP32 1024-point three-component
+    // row, whose passes then hold seven blocks per SM), else 256
+    static constexpr int NT = (NC * ROWS * M >= 1024 && !(F32 && NX == 1024)) ? 256 : 128;
     // FP32 forward passes: ask the register allocator for 8 resident 128-thread
     // blocks per SM (64 registers), so that enough loads are in flight, on the
     // sizes where the tangent of the mechanics pass fits without spilling; the
     // 512-point three-component pass takes 9 (56 registers, 8 bytes of spill:
-    // measured 0.7 % faster in the concurrent-stream launch mode)
-    static constexpr int MINB = (sizeof(T) == 4 && (NX == 128 || NX == 512 || NX == 1024))
-                                    ? (NX == 512 && NC == 3 ? 9 : 8) * 128 / NT : 1;
-    // FP32 512-point inverse passes: 7 resident blocks per SM (72 registers; 16-40 bytes of
-    // spill in the update kernels), measured faster than 6 blocks at 80 registers and 5 at 96
-    // when the one- and three-component passes of concurrent simulations share the SMs (8 at 64
-    // registers spills 72 bytes and was slower)
-    static constexpr int MINB_INV = (sizeof(T) == 4 && NX == 512) ? 7 : 1;
+    // measured 0.7 % faster in the concurrent-stream launch mode), the 2048-point
+    // one-component pass 5 of 256 threads (BCCG direction 24.1 -> 22.1 us)
+    static constexpr int MINB = !F32 ? 1
+                                : NX == 128 || NX == 512 || NX == 1024 ? (NX == 512 && NC == 3 ? 9 : 8)
+                                : NX == 2048 && NC == 1                ? 5
+                                                                       : 1;
+    // FP32 inverse passes of 256 points on take their epilogue's loads a few pixels at a time after
+    // the FFT and ask for enough resident blocks to overlap it with other blocks' transforms, instead
+    // of prefetching all of a thread's pixels (up to 8, 70 registers) before it: one launch with every
+    // problem active, us, prefetching -> here: CG update 2048^2 143 -> 80, 1024^2 36 -> 25, eight 512^2
+    // 22.5 -> 20.3; BCCG iterate 2048^2 85 -> 66, 1024^2 31 -> 27, one 512^2 21 -> 18, eight 40 -> 35.
+    // (Fewer blocks: 2048-point iterate at 2 blocks 79 us; more: spills, 4 blocks 71 us; 512 threads 81.)
+    static constexpr int PREFETCH = F32 && NX >= 256 ? 2 : 8;   // most pixels per thread that are prefetched
+    static constexpr int MINB_INV = !F32 ? 1
+                                    : NX == 2048 ? (NC == 3 ? 4 : 3)
+                                    : NX == 1024 ? 7
+                                    : NX == 512  ? (NC == 3 ? 9 : 7)
+                                    : NX == 256  ? (NC == 3 ? 10 : 6)
+                                                 : 1;
     static constexpr int SP = padded_len(M) + 2;            // pitch (complex): padded M values + slot for k = M
     static constexpr int NSEQ = NC * ROWS;
     // twiddles staged in shared memory: length-M FFT table (padded indices) + the
@@ -257,11 +271,6 @@ __device__ __forceinline__ int ridx(int x) { return 2 * pidx(x >> 1) + (x & 1); 
 //   static void finalize(const Desc<T>&, const double (&tot)[NR]);   // one thread
 #ifndef PFF_ROW_G
 #define PFF_ROW_G 2
-#endif
-// Row-inverse passes issue the epilogue's pixel loads before staging and transforming the
-// spectrum (they land during the FFT) when a thread handles at most this many pixels.
-#ifndef PFF_INV_PREFETCH
-#define PFF_INV_PREFETCH 8
 #endif
 template <class F, bool TWO> struct InOf { struct type {}; };
 template <class F> struct InOf<F, true> { using type = typename F::In; };
@@ -397,8 +406,8 @@ __global__ void __launch_bounds__(RowCfg<T, NX, NC>::NT) k_row_fwd_u(const Desc<
     row_fwd_body<T, NX, NC, F>(descs);
 }
 
-// Row-inverse pass of one row group y0: the epilogue's pixel loads are issued
-// first (they land during the staging and the FFT), the half-spectrum rows are
+// Row-inverse pass of one row group y0: a few pixels' epilogue loads are issued
+// first (they land during the staging and the FFT; see PREFETCH), the half-spectrum rows are
 // staged, combined for the complex-to-real transform, transformed back along x,
 // and the epilogue runs on the real values (accumulating F's reductions in acc).
 template <typename T, int NX, int NC, class F>
@@ -408,7 +417,7 @@ __device__ __forceinline__ void row_inv_item(const Desc<T>& d, const typename F:
     using C = typename CT<T>::t;
     constexpr int M = Cfg::M, SP = Cfg::SP, ROWS = Cfg::ROWS, NT = Cfg::NT;
     const T* rb = reinterpret_cast<const T*>(buf);
-    constexpr bool TWO = HasIn<F>::value && (ROWS * NX) % NT == 0 && ROWS * NX / NT <= PFF_INV_PREFETCH;
+    constexpr bool TWO = HasIn<F>::value && (ROWS * NX) % NT == 0 && ROWS * NX / NT <= Cfg::PREFETCH;
     constexpr int PPT = TWO ? ROWS * NX / NT : 1;
     using InT = typename InOf<F, TWO>::type;
     InT in[PPT];
@@ -467,6 +476,29 @@ __device__ __forceinline__ void row_inv_item(const Desc<T>& d, const typename F:
 #pragma unroll
             for (int c = 0; c < NC; ++c) v[c] = rb[(c * ROWS + row) * 2 * SP + ridx(x)];
             F::pixel(d, ctx, (size_t)((unsigned)(y0 + row) * NX + x), in[j], v, acc);
+        }
+    } else if constexpr (HasIn<F>::value && (ROWS * NX) % NT == 0) {
+        (void)in;
+        // the loads of a few pixels at a time (about 32 registers) are in flight together
+        constexpr int N = ROWS * NX / NT, WORDS = (int)((sizeof(typename F::In) + 3) / 4);
+        constexpr int G = pow2floor(cmin(N, cmax(2, 32 / WORDS)));
+#pragma unroll 1
+        for (int j0 = 0; j0 < N; j0 += G) {
+            typename F::In b[G];
+#pragma unroll
+            for (int j = 0; j < G; ++j) {
+                const int t = threadIdx.x + (j0 + j) * NT;
+                b[j] = F::load(d, ctx, (size_t)((unsigned)(y0 + t / NX) * NX + t % NX));
+            }
+#pragma unroll
+            for (int j = 0; j < G; ++j) {
+                const int t = threadIdx.x + (j0 + j) * NT;
+                const int row = t / NX, x = t % NX;
+                T v[NC];
+#pragma unroll
+                for (int c = 0; c < NC; ++c) v[c] = rb[(c * ROWS + row) * 2 * SP + ridx(x)];
+                F::pixel(d, ctx, (size_t)((unsigned)(y0 + row) * NX + x), b[j], v, acc);
+            }
         }
     } else {
         (void)in;
