@@ -1446,6 +1446,7 @@ int pff_solve_mechanics(pff_problem* h, pff_step_report* out) {
     Group g = single_group(h);
     const pff_params& p = h->prm;
     int rc;
+    bool warmed = h->graphs.exec[0] || h->graphs.exec[1];
     auto body = [&](auto tag) -> int {
         using T = decltype(tag);
         const Desc<T>* d = (const Desc<T>*)h->d_desc;
@@ -1454,7 +1455,7 @@ int pff_solve_mechanics(pff_problem* h, pff_step_report* out) {
         for (int round = 0; round <= p.mech_max_newton; ++round) {
             run_trio<T>(h, RF_NEWTON, CO_GAMMA_N, RI_NEWTON);
             for (int it = 0; it <= p.mech_max_cg + CHUNK; it += CHUNK) {
-                chunk_direct<T>(0, g);
+                run_chunk<T>(0, g, warmed);
                 int r2 = poll<T>(g, false, h);
                 if (r2) return r2;
                 if (all_bits(g, 1)) break;
@@ -1485,6 +1486,7 @@ int pff_solve_phase_field(pff_problem* h, pff_step_report* out) {
         if (e != cudaSuccess) return cuda_fail(h, e, "phase-field update");
         return h->prec == PFF_FP64 ? poll<double>(g, true, h) : poll<float>(g, true, h);
     };
+    bool warmed = h->graphs.exec[0] || h->graphs.exec[1];
     // rescale disabled for a bare sub-problem: gamma = 1
     auto body = [&](auto tag) -> int {
         using T = decltype(tag);
@@ -1508,7 +1510,7 @@ int pff_solve_phase_field(pff_problem* h, pff_step_report* out) {
         }
         if (!resident_solve<T>(1, g)) {
             for (int c = bccg_chunks(g, p.pf_max_iter); c > 0; --c) {
-                chunk_direct<T>(1, g);
+                run_chunk<T>(1, g, warmed);
                 int r2 = poll<T>(g, false, h);
                 if (r2) return r2;
                 if (all_bits(g, 4)) break;
