@@ -5,6 +5,8 @@
 #include <cuda_runtime.h>
 #include <stdint.h>
 
+#include <type_traits>
+
 namespace pff {
 
 // ---------------------------------------------------------------------------
@@ -136,17 +138,17 @@ __device__ __forceinline__ void pdl_enter() { pdl_wait(); pdl_release(); }
 // Per-block constants: thread 0 evaluates F::skip and F::prep once (control
 // block loads and FP64-to-FP32 conversions, which run on GB300's narrow FP64
 // pipe) and shares the result through shared memory.  Returns true when the
-// whole problem is skipped.  Ctx must be trivially copyable.
+// whole problem is skipped.  Ctx must be trivially copyable.  prep does not wait
+// for the skip test: its loads and the flag's (some 700 cycles from L2) overlap.
 template <class F, class D, class X>
 __device__ __forceinline__ bool block_prep(const D& d, X& ctx) {
     __shared__ __align__(16) unsigned char s_raw[sizeof(X)];
     __shared__ int s_skip;
     if (threadIdx.x == 0) {
-        s_skip = F::skip(d) ? 1 : 0;
-        if (!s_skip) {
-            const X c = F::prep(d);
-            memcpy(s_raw, &c, sizeof(X));
-        }
+        const int skip = F::skip(d) ? 1 : 0;
+        const X c = F::prep(d);
+        memcpy(s_raw, &c, sizeof(X));
+        s_skip = skip;
     }
     __syncthreads();
     if (s_skip) return true;
@@ -163,7 +165,7 @@ __device__ __forceinline__ double ldd(const double* p) { return __ldcg(p); }
 // Per-thread accumulation.  FP64 problems accumulate in double.  FP32 problems
 // accumulate products exactly split (fmaf) and summed with Knuth's two-sum in
 // a float pair, and reduce across the grid in double-float arithmetic
-// (reduce_grid): the work stays on the FP32 pipe while the sums keep close to
+// (reduce_finalize): the work stays on the FP32 pipe while the sums keep close to
 // FP64 accuracy.
 // Functors whose per-pixel work splits into load() (returning an In record) and
 // pixel(..., const In&, ...) let a kernel issue the loads of all of a thread's
@@ -177,7 +179,7 @@ __device__ __forceinline__ void pixel_one(const D& d, const X& c, size_t i, A&&.
     else F::pixel(d, c, i, a...);
 }
 
-struct DF { float hi, lo; };   // double-float value hi + lo (see reduce_grid)
+struct DF { float hi, lo; };   // double-float value hi + lo (see reduce_finalize)
 template <typename T> struct Acc;
 // count(x): a small integer (a pixel count); a thread's sum of counts is exact in
 // either precision (below 2^24), so it needs no compensation.
@@ -211,10 +213,9 @@ template <> struct Acc<float> {
     }
 };
 
-// Grid reductions.  Each block reduces its threads' values (warp shuffles, then
-// one shuffle tree over the warp totals in warp 0) into part[blockIdx.x*NR + k];
-// the last block of the problem (by an atomic ticket) sums all partials in a
-// fixed order and returns true with the totals in tot (valid in thread 0).
+// Grid reductions.  Each block reduces its threads' values (a shuffle tree per value) into
+// part[blockIdx.x*NR + k]; the last block of the problem (by an atomic ticket) sums all partials in a
+// fixed order, the totals in tot (valid in thread 0), and runs the finalizer (reduce_finalize).
 // Deterministic: the summation tree depends only on the grid shape.
 //
 // FP32 problems: every product is formed exactly (fmaf split), each thread's
@@ -222,7 +223,7 @@ template <> struct Acc<float> {
 // double-float arithmetic (a value is an unevaluated sum hi + lo of two floats,
 // added with Knuth's two-sum; about 44 significant bits) so that the per-pixel
 // and per-thread work stays on the FP32 pipe; the block totals and the
-// cross-block sum are FP64 (reduce_grid).
+// cross-block sum are FP64 (reduce_finalize).
 __device__ __forceinline__ DF df_add(DF a, DF b) {
     float s = a.hi + b.hi;
     float z = s - a.hi;
@@ -270,8 +271,6 @@ template <> struct RedOps<double> {
     __device__ static double zero() { return 0.0; }
     __device__ static double add(double a, double b) { return a + b; }
     __device__ static double shfl(double a, int o) { return __shfl_down_sync(0xffffffffu, a, o); }
-    __device__ static void store(double* part, size_t j, double v) { __stcg(part + j, v); }
-    __device__ static double load(const double* part, size_t j) { return __ldcg(part + j); }
     __device__ static double total(double v) { return v; }
 };
 template <> struct RedOps<DF> {
@@ -280,26 +279,18 @@ template <> struct RedOps<DF> {
     __device__ static DF shfl(DF a, int o) {
         return DF{__shfl_down_sync(0xffffffffu, a.hi, o), __shfl_down_sync(0xffffffffu, a.lo, o)};
     }
-    __device__ static void store(double* part, size_t j, DF v) {
-        __stcg(reinterpret_cast<float2*>(part) + j, make_float2(v.hi, v.lo));
-    }
-    __device__ static DF load(const double* part, size_t j) {
-        float2 y = __ldcg(reinterpret_cast<const float2*>(part) + j);
-        return DF{y.x, y.y};
-    }
     __device__ static double total(DF v) { return (double)v.hi + (double)v.lo; }
 };
 
 // Block reduction in a fixed order: every thread stores its NR values in shared
 // memory, then warp w reduces values k = w, w + NW, ... (lane l adds entries
 // l, l + 32, ... in order, then a shuffle tree), so that each value costs one
-// warp's tree instead of a tree in every warp.  res is valid in thread 0.
+// warp's tree instead of a tree in every warp.  The totals are left in res.
 template <int NR, int NT, typename V>
 __device__ __forceinline__ void block_reduce(const V (&v)[NR], V (&res)[NR]) {
     using O = RedOps<V>;
     constexpr int NW = NT / 32;
     __shared__ V sh[NR][NT];
-    __shared__ V shr[NR];
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int k = 0; k < NR; ++k) sh[k][threadIdx.x] = v[k];
@@ -310,68 +301,99 @@ __device__ __forceinline__ void block_reduce(const V (&v)[NR], V (&res)[NR]) {
         for (int j = 1; j < NW; ++j) x = O::add(x, sh[k][lane + 32 * j]);
 #pragma unroll
         for (int o = 16; o > 0; o >>= 1) x = O::add(x, O::shfl(x, o));
-        if (lane == 0) shr[k] = x;
+        if (lane == 0) res[k] = x;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int k = 0; k < NR; ++k) res[k] = shr[k];
-    }
 }
 
 // The cross-block stage is FP64 for both precisions: each block's total is stored
 // as one double (a double-float pair hi + lo converts exactly), and the last block
 // sums the partials in double.  Within a block an FP32 problem's values stay
 // double-float pairs (FP32 pipe); an FP64 problem's stay doubles.
-template <int NR, int NT, typename V>
-__device__ __forceinline__ bool reduce_grid(V (&v)[NR], double* part, unsigned* counter, int nblocks,
-                                            double (&tot)[NR]) {
-    using O = RedOps<V>;
+//
+// This tail is a serial chain at the end of a kernel: an L2 round trip takes 700 to 900 cycles and an
+// FP64 operation 65.  So the block's values are converted and stored by one lane each; the last
+// block's threads hold one value each of several blocks and load them eight at a time; and the
+// control block and the descriptor, which the finalizer works on, come into shared memory beside the
+// partials and go back in one go.  (Eight values of the 512^2 BCCG iterate: 19000 of the kernel's 30000
+// cycles lay between its last pixel and its end with one thread storing, a load at a time and the
+// finalizer on global memory: 18.7 us, now 14.6; 2048^2 66 -> 60 us.)
+constexpr int red_lanes(int n) { return n <= 1 ? 1 : n <= 2 ? 2 : n <= 4 ? 4 : 8; }
+
+// Block and grid reduction of the per-thread accumulators, F::finalize(descriptor, totals) in the last block.
+template <class F, int NR, int NT, typename T>
+__device__ __forceinline__ void reduce_finalize(const Acc<T>* acc, const Desc<T>& d, int nblocks) {
+    using V = typename std::conditional<sizeof(T) == 4, DF, double>::type;
+    static_assert(NR >= 1 && NR <= 8 && NT >= 64, "one lane per value");
+    constexpr int KP = red_lanes(NR), NW = NT / 32, S = NT / KP;   // S blocks per pass
+    constexpr int CWORDS = (int)(sizeof(Ctrl) / 4), DWORDS = (int)(sizeof(Desc<T>) / 4);
+    __shared__ V bs[NR];
+    __shared__ double shw[NW][KP];
+    __shared__ __align__(16) int s_ctrl[CWORDS];
+    __shared__ __align__(16) int s_desc[DWORDS];
     __shared__ int s_last;
-    V bs[NR];
-    block_reduce<NR, NT>(v, bs);
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int k = 0; k < NR; ++k) __stcg(part + (size_t)blockIdx.x * NR + k, O::total(bs[k]));
-        __threadfence();
-        unsigned t = atomicAdd(counter, 1u);
-        s_last = (t == (unsigned)(nblocks - 1));
-    }
-    __syncthreads();
-    if (!s_last) return false;
-    __threadfence();
-    // fixed-order FP64 sum of the partials: thread t takes blocks t, t+NT, ... in order
-    double x[NR];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    V v[NR];
 #pragma unroll
     for (int k = 0; k < NR; ++k) {
-        x[k] = 0.0;
-        for (int b = threadIdx.x; b < nblocks; b += NT) x[k] += __ldcg(part + (size_t)b * NR + k);
+        if constexpr (sizeof(T) == 4) v[k] = acc[k].df();
+        else v[k] = acc[k].get();
     }
-    double tt[NR];
-    block_reduce<NR, NT>(x, tt);
-    if (threadIdx.x == 0) {
-#pragma unroll
-        for (int k = 0; k < NR; ++k) tot[k] = tt[k];
-        *counter = 0u;
+    block_reduce<NR, NT>(v, bs);
+    if (warp == 0) {
+        if (lane < NR) __stcg(d.part + (size_t)blockIdx.x * NR + lane, RedOps<V>::total(bs[lane]));
+        __threadfence();
+        __syncwarp();
+        if (lane == 0) s_last = atomicAdd(&d.ctrl->counter, 1u) == (unsigned)(nblocks - 1);
     }
-    return true;
-}
-
-// Block + grid reduction of the per-thread accumulators.
-template <int NR, int NT, typename T>
-__device__ __forceinline__ bool reduce_acc(const Acc<T>* acc, double* part, unsigned* counter, int nblocks,
-                                           double (&tot)[NR]) {
-    if constexpr (sizeof(T) == 4) {
-        DF v[NR];
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    const int* gc = reinterpret_cast<const int*>(d.ctrl);
+    const int* gd = reinterpret_cast<const int*>(&d);
+    for (int w = tid; w < CWORDS; w += NT) s_ctrl[w] = __ldcg(gc + w);
+    for (int w = tid; w < DWORDS; w += NT) s_desc[w] = gd[w];
+    // thread (b0, k) sums value k of the blocks b0, b0 + S, ...
+    const int k = tid % KP;
+    double x = 0.0;
+    for (int b = tid / KP; b < nblocks; b += 8 * S) {
+        double y[8];
 #pragma unroll
-        for (int k = 0; k < NR; ++k) v[k] = acc[k].df();
-        return reduce_grid<NR, NT>(v, part, counter, nblocks, tot);
-    } else {
-        double v[NR];
-#pragma unroll
-        for (int k = 0; k < NR; ++k) v[k] = acc[k].get();
-        return reduce_grid<NR, NT>(v, part, counter, nblocks, tot);
+        for (int u = 0; u < 8; ++u) {
+            const int bb = b + u * S;
+            y[u] = k < NR && bb < nblocks ? __ldcg(d.part + (size_t)bb * NR + k) : 0.0;
+        }
+        x += ((y[0] + y[1]) + (y[2] + y[3])) + ((y[4] + y[5]) + (y[6] + y[7]));
     }
+#pragma unroll
+    for (int o = KP; o < 32; o *= 2) x += __shfl_xor_sync(0xffffffffu, x, o);
+    if (lane < KP) shw[warp][lane] = x;
+    __syncthreads();
+    if (warp == 0) {
+        if (lane < KP) {
+            double t[NW];
+#pragma unroll
+            for (int w = 0; w < NW; ++w) t[w] = shw[w][lane];
+#pragma unroll
+            for (int n = 1; n < NW; n *= 2)
+#pragma unroll
+                for (int w = 0; w + n < NW; w += 2 * n) t[w] += t[w + n];
+            shw[0][lane] = t[0];
+        }
+        __syncwarp();
+        if (lane == 0) {
+            double tot[NR];
+#pragma unroll
+            for (int q = 0; q < NR; ++q) tot[q] = shw[0][q];
+            Desc<T>& sd = *reinterpret_cast<Desc<T>*>(s_desc);
+            sd.ctrl = reinterpret_cast<Ctrl*>(s_ctrl);
+            F::finalize(sd, tot);
+            sd.ctrl->counter = 0u;
+        }
+    }
+    __syncthreads();
+    int* out = reinterpret_cast<int*>(d.ctrl);
+    for (int w = tid; w < CWORDS; w += NT) __stcg(out + w, s_ctrl[w]);
 }
 
 // ---------------------------------------------------------------------------

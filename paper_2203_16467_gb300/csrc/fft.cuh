@@ -383,11 +383,7 @@ __device__ __forceinline__ void row_fwd_body(const Desc<T>* __restrict__ descs) 
     constexpr int NRA = F::NR > 0 ? F::NR : 1;
     Acc<T> acc[NRA];
     row_fwd_pixels<T, NX, NC, F>(d, ctx, y0, buf, &acc[0]);
-    if constexpr (F::NR > 0) {
-        double tot[F::NR];
-        if (reduce_acc<F::NR, NT>(acc, d.part, &d.ctrl->counter, gridDim.x, tot) && threadIdx.x == 0)
-            F::finalize(d, tot);
-    }
+    if constexpr (F::NR > 0) reduce_finalize<F, F::NR, NT>(acc, d, gridDim.x);
     cp_async_wait_all();
     __syncthreads();
     row_fwd_fft_store<T, NX, NC>(d, y0, buf, tws);
@@ -530,11 +526,7 @@ __device__ __forceinline__ void row_inv_body(const Desc<T>* __restrict__ descs) 
     constexpr int NRA = F::NR > 0 ? F::NR : 1;
     Acc<T> acc[NRA];
     row_inv_item<T, NX, NC, F>(d, ctx, blockIdx.x * Cfg::ROWS, buf, tws, &acc[0]);
-    if constexpr (F::NR > 0) {
-        double tot[F::NR];
-        if (reduce_acc<F::NR, NT>(acc, d.part, &d.ctrl->counter, gridDim.x, tot) && threadIdx.x == 0)
-            F::finalize(d, tot);
-    }
+    if constexpr (F::NR > 0) reduce_finalize<F, F::NR, NT>(acc, d, gridDim.x);
 }
 template <typename T, int NX, int NC, class F>
 __global__ void __launch_bounds__(RowCfg<T, NX, NC>::NT, RowCfg<T, NX, NC>::MINB_INV) k_row_inv(const Desc<T>* __restrict__ descs) {
@@ -615,11 +607,7 @@ __global__ void __launch_bounds__(ColCfg<T, NY, NC>::NT) k_col(const Desc<T>* __
         const int j = t % CW, ky = (t / CW) % NY, c = t / (CW * NY);
         d.S[c * plane + (unsigned)ky * d.wp + kx0 + j] = buf[(c * CW + j) * SP + pidx(ky)];
     }
-    if constexpr (ColNR<OP>::value > 0) {
-        double tot[ColNR<OP>::value];
-        if (reduce_acc<ColNR<OP>::value, NT>(acc, d.part, &d.ctrl->counter, gridDim.x, tot) && threadIdx.x == 0)
-            OP::finalize(d, tot);
-    }
+    if constexpr (ColNR<OP>::value > 0) reduce_finalize<OP, ColNR<OP>::value, NT>(acc, d, gridDim.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -759,12 +747,7 @@ __global__ void __launch_bounds__(64 * CW) k_col512(const Desc<T>* __restrict__ 
     constexpr int NRA = ColNR<OP>::value > 0 ? ColNR<OP>::value : 1;
     Acc<T> acc[NRA];
     col512_item<T, NC, OP, CW>(d, mk, blockIdx.x * CW, xb, tws, acc);
-    if constexpr (ColNR<OP>::value > 0) {
-        double tot[ColNR<OP>::value];
-        if (reduce_acc<ColNR<OP>::value, 64 * CW>(acc, d.part, &d.ctrl->counter, gridDim.x, tot) &&
-            threadIdx.x == 0)
-            OP::finalize(d, tot);
-    }
+    if constexpr (ColNR<OP>::value > 0) reduce_finalize<OP, ColNR<OP>::value, 64 * CW>(acc, d, gridDim.x);
 }
 
 // ---------------------------------------------------------------------------
@@ -941,11 +924,7 @@ __global__ void __launch_bounds__(CW * NY / 16, NC == 1 && NY == 2048 ? 2 : 1) k
 #pragma unroll
         for (int m = 0; m < 16; ++m) S[c * plane + m * step] = u[c][at16(m)];
     }
-    if constexpr (ColNR<OP>::value > 0) {
-        double tot[ColNR<OP>::value];
-        if (reduce_acc<ColNR<OP>::value, Cfg::NT>(acc, d.part, &d.ctrl->counter, gridDim.x, tot) && threadIdx.x == 0)
-            OP::finalize(d, tot);
-    }
+    if constexpr (ColNR<OP>::value > 0) reduce_finalize<OP, ColNR<OP>::value, Cfg::NT>(acc, d, gridDim.x);
 }
 
 // ---------------------------------------------------------------------------

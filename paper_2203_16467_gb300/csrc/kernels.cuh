@@ -40,11 +40,7 @@ __global__ void __launch_bounds__(EL_NT) k_elem(const Desc<T>* __restrict__ desc
     constexpr int NRA = F::NR > 0 ? F::NR : 1;
     Acc<T> acc[NRA];
     elem_items<T, F>(d, ctx, &acc[0]);
-    if constexpr (F::NR > 0) {
-        double tot[F::NR];
-        if (reduce_acc<F::NR, EL_NT>(acc, d.part, &d.ctrl->counter, gridDim.x, tot) && threadIdx.x == 0)
-            F::finalize(d, tot);
-    }
+    if constexpr (F::NR > 0) reduce_finalize<F, F::NR, EL_NT>(acc, d, gridDim.x);
 }
 
 // Reset of the per-step solver state (one thread per problem).
