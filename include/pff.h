@@ -371,9 +371,8 @@ int pff_batch_autotune(pff_batch* b, const int* group_sizes, int n_candidates, i
  * synchronisation an allocation may cause.
  *   out_dev = nabla^2_N in_dev on an nx x ny periodic grid of spacing dx, both
  *   FP64 device arrays of nx*ny values (row-major, y slow), owned by the caller.
- * Scratch (one half spectrum, about 2.2 MB), twiddle table and kernel
- * descriptor are static device arrays that every GPU loading the library holds
- * until the process exits.  The first call on a device sets them up (with that
+ * Scratch (one half spectrum, about 2.2 MB) and twiddle table are static device
+ * arrays that every GPU loading the library holds until the process exits.  The first call on a device sets them up (with that
  * device current): make that first call before any stream capture.  Calls
  * share the arrays, so calls whose kernels overlap on the GPU (different
  * streams, or different host threads) race; serialise them.  Nothing in the

@@ -54,8 +54,8 @@ def build(force=False, verbose=False, jobs=None):
     for host_tu in ("api.cu", "noalloc.cu", "micro.cu"):
         jobs_list.append([cc, *ARCH, *FLAGS, "-c", os.path.join(CSRC, host_tu),
                           "-o", os.path.join(BUILD, host_tu.replace(".cu", ".o"))])
-    # the cluster-resident solves of small grids (FP32 only; one object per solve)
-    for kind, tag in enumerate(("mech", "bccg")):
+    # the cluster-resident solves of small grids and their Laplacian (FP32 only; one object each)
+    for kind, tag in enumerate(("mech", "bccg", "lap")):
         jobs_list.append([cc, *ARCH, *FLAGS, "-DPFF_REAL=float", f"-DPFF_RESIDENT={kind}", "-c",
                           os.path.join(CSRC, "k_resident.cu"), "-o", os.path.join(BUILD, f"k_resident_{tag}.o")])
     # the cluster mechanics solve (FP32 only)

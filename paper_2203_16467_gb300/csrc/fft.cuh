@@ -365,11 +365,10 @@ __device__ __forceinline__ void stage_row_twiddles(const Desc<T>& d, typename CT
 }
 
 template <typename T, int NX, int NC, class F>
-__device__ __forceinline__ void row_fwd_body(const Desc<T>* __restrict__ descs) {
+__device__ __forceinline__ void row_fwd_body(const Desc<T>& d) {
     using Cfg = RowCfg<T, NX, NC>;
     using C = typename CT<T>::t;
     constexpr int NT = Cfg::NT;
-    const Desc<T>& d = descs[blockIdx.y];
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* buf = reinterpret_cast<C*>(smem_raw);
     C* tws = buf + Cfg::NSEQ * Cfg::SP;
@@ -395,11 +394,11 @@ __device__ __forceinline__ void row_fwd_body(const Desc<T>* __restrict__ descs) 
 // no bound to ptxas, which then takes more registers).
 template <typename T, int NX, int NC, class F>
 __global__ void __launch_bounds__(RowCfg<T, NX, NC>::NT, RowCfg<T, NX, NC>::MINB) k_row_fwd(const Desc<T>* __restrict__ descs) {
-    row_fwd_body<T, NX, NC, F>(descs);
+    row_fwd_body<T, NX, NC, F>(descs[blockIdx.y]);
 }
 template <typename T, int NX, int NC, class F>
 __global__ void __launch_bounds__(RowCfg<T, NX, NC>::NT) k_row_fwd_u(const Desc<T>* __restrict__ descs) {
-    row_fwd_body<T, NX, NC, F>(descs);
+    row_fwd_body<T, NX, NC, F>(descs[blockIdx.y]);
 }
 
 // Row-inverse pass of one row group y0: a few pixels' epilogue loads are issued
@@ -511,11 +510,10 @@ __device__ __forceinline__ void row_inv_item(const Desc<T>& d, const typename F:
 }
 
 template <typename T, int NX, int NC, class F>
-__device__ __forceinline__ void row_inv_body(const Desc<T>* __restrict__ descs) {
+__device__ __forceinline__ void row_inv_body(const Desc<T>& d) {
     using Cfg = RowCfg<T, NX, NC>;
     using C = typename CT<T>::t;
     constexpr int NT = Cfg::NT;
-    const Desc<T>& d = descs[blockIdx.y];
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* buf = reinterpret_cast<C*>(smem_raw);
     C* tws = buf + Cfg::NSEQ * Cfg::SP;
@@ -530,11 +528,11 @@ __device__ __forceinline__ void row_inv_body(const Desc<T>* __restrict__ descs) 
 }
 template <typename T, int NX, int NC, class F>
 __global__ void __launch_bounds__(RowCfg<T, NX, NC>::NT, RowCfg<T, NX, NC>::MINB_INV) k_row_inv(const Desc<T>* __restrict__ descs) {
-    row_inv_body<T, NX, NC, F>(descs);
+    row_inv_body<T, NX, NC, F>(descs[blockIdx.y]);
 }
 template <typename T, int NX, int NC, class F>
 __global__ void __launch_bounds__(RowCfg<T, NX, NC>::NT) k_row_inv_u(const Desc<T>* __restrict__ descs) {
-    row_inv_body<T, NX, NC, F>(descs);
+    row_inv_body<T, NX, NC, F>(descs[blockIdx.y]);
 }
 
 // Column pass: CWE adjacent columns kx of the half spectrum, all NC planes.
@@ -562,11 +560,10 @@ struct ColPrep {
 };
 
 template <typename T, int NY, int NC, class OP>
-__global__ void __launch_bounds__(ColCfg<T, NY, NC>::NT) k_col(const Desc<T>* __restrict__ descs) {
+__device__ __forceinline__ void col_body(const Desc<T>& d) {
     using Cfg = ColCfg<T, NY, NC>;
     using C = typename CT<T>::t;
     constexpr int CW = Cfg::CWE, SP = Cfg::SP, NT = Cfg::NT;
-    const Desc<T>& d = descs[blockIdx.y];
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* buf = reinterpret_cast<C*>(smem_raw);
     pdl_enter();
@@ -608,6 +605,10 @@ __global__ void __launch_bounds__(ColCfg<T, NY, NC>::NT) k_col(const Desc<T>* __
         d.S[c * plane + (unsigned)ky * d.wp + kx0 + j] = buf[(c * CW + j) * SP + pidx(ky)];
     }
     if constexpr (ColNR<OP>::value > 0) reduce_finalize<OP, ColNR<OP>::value, NT>(acc, d, gridDim.x);
+}
+template <typename T, int NY, int NC, class OP>
+__global__ void __launch_bounds__(ColCfg<T, NY, NC>::NT) k_col(const Desc<T>* __restrict__ descs) {
+    col_body<T, NY, NC, OP>(descs[blockIdx.y]);
 }
 
 // ---------------------------------------------------------------------------
@@ -733,10 +734,9 @@ __device__ __forceinline__ void col512_item(const Desc<T>& d, const ModeK<T>& mk
         for (int e = 0; e < 8; ++e) d.S[c * plane + (unsigned)(tp + 64 * e) * d.wp + kx] = u[c][e];
 }
 
-template <typename T, int NC, class OP, int CW = COL512_CW>
-__global__ void __launch_bounds__(64 * CW) k_col512(const Desc<T>* __restrict__ descs) {
+template <typename T, int NC, class OP, int CW>
+__device__ __forceinline__ void col512_body(const Desc<T>& d) {
     using C = typename CT<T>::t;
-    const Desc<T>& d = descs[blockIdx.y];
     extern __shared__ __align__(16) unsigned char smem_raw[];
     C* tws = reinterpret_cast<C*>(smem_raw);
     C* xb = tws + padded_len(512);
@@ -748,6 +748,10 @@ __global__ void __launch_bounds__(64 * CW) k_col512(const Desc<T>* __restrict__ 
     Acc<T> acc[NRA];
     col512_item<T, NC, OP, CW>(d, mk, blockIdx.x * CW, xb, tws, acc);
     if constexpr (ColNR<OP>::value > 0) reduce_finalize<OP, ColNR<OP>::value, 64 * CW>(acc, d, gridDim.x);
+}
+template <typename T, int NC, class OP, int CW = COL512_CW>
+__global__ void __launch_bounds__(64 * CW) k_col512(const Desc<T>* __restrict__ descs) {
+    col512_body<T, NC, OP, CW>(descs[blockIdx.y]);
 }
 
 // ---------------------------------------------------------------------------

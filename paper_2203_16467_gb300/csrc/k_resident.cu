@@ -44,9 +44,7 @@
 // private copy of the control block in each CTA's shared memory takes the finalizers' results and
 // rank 0 stores it at the end.  Sums: compensated pairs per thread, double-float within a CTA,
 // FP64 across the CTAs in a fixed order.
-#include <map>
-#include <mutex>
-#include <utility>
+#include <atomic>
 
 #include "kernels.cuh"
 #include "launch.h"
@@ -895,57 +893,114 @@ __global__ void __launch_bounds__(RG<NX, NY, 1>::NT, 1) k_res_bccg(const Desc<fl
     leave<G>(d, s, t.rank);
 }
 
+// ---------------------------------------------------------------- one Laplacian
+// out = nabla^2 in of one field, in = d.r[0], out = d.q[0] (the allocation-free entry point): the
+// operator alone, without the scalar warp.  A wait that runs out leaves NaN, never a wrong field.
+// Bound by its two exchanges and the launch: everything that does not depend on the input (twiddles,
+// lane constants, the cluster's start) runs before the wait for the stream's previous work.  Per call in
+// a row of calls, three passes -> one launch (without the overlap): 16^2 6.1 -> 2.7 us (4.1), 64^2 6.1 ->
+// 2.7 us (6.2), 128^2 7.0 -> 3.7 us (6.2), 256 x 64 7.3 -> 4.0 us (6.2).
+template <int NX, int NY>
+__global__ void __launch_bounds__(RG<NX, NY, 1>::W * 32, 1) k_res_lap(const __grid_constant__ Desc<float> d) {
+    using G = RG<NX, NY, 1>;
+    constexpr int E = G::ER;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ Shared s;
+    C* sm = reinterpret_cast<C*>(smem_raw);
+    if (threadIdx.x == 0) {
+        s.dead = 0;
+        for (int b = 0; b < 4; ++b) bar_init(s32(&s.bar[b]));
+        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+    }
+    Lane<G> t;
+    lane_setup<NX, NY, 1>(t, d, s, sm);
+    const unsigned pix = (t.rank * G::RPC + t.row) * NX + 2 * t.li;
+    C z[E];
+    for (int i = threadIdx.x; i < NY; i += G::W * 32) sm[G::O_TWC + i] = d.tw[NY + i];
+    const ModeK<float> mk(d);
+    __syncthreads();
+    cluster_sync_all();
+    pdl_enter();   // the stream's previous work is complete from here on
+#pragma unroll
+    for (int e = 0; e < E; ++e)
+        z[e] = t.on ? *reinterpret_cast<const C*>(d.r[0] + pix + e * 2 * G::LR) : C{0.f, 0.f};
+    unsigned par = 0;
+    operate<NX, NY, 1, FColLapPlain>(t, s, sm, mk, z, par, nullptr, [] {});
+    __syncthreads();
+    const bool dead = s.dead;
+    if (t.on) {
+#pragma unroll
+        for (int e = 0; e < E; ++e)
+            *reinterpret_cast<C*>(d.q[0] + pix + e * 2 * G::LR) = dead ? C{NAN, NAN} : z[e];
+    }
+    if (dead) {
+        const long long t0 = clock64();
+        while (clock64() - t0 < 1000000) {}
+    }
+    cluster_sync_all();
+}
+
 // ---------------------------------------------------------------- launch
 // One cluster of CS CTAs per problem.  cudaErrorNotSupported where the device cannot host the
-// cluster (the caller then runs the per-kernel path).
-cudaError_t go(void (*fn)(const Desc<float>*), int cs, int nt, size_t smem, const Desc<float>* d, int np,
-               cudaStream_t st) {
-    static std::mutex mu;
-    static std::map<std::pair<const void*, int>, bool> known;   // (kernel, device) -> can run
+// cluster (the caller then runs the per-kernel path).  pdl: may be scheduled while the stream's
+// previous kernel runs.
+constexpr int MAX_DEVICES = 64;
+enum : signed char { UNKNOWN = 0, RUNS = 1, REFUSED = 2 };
+template <typename A>
+cudaError_t go(void (*fn)(A), std::atomic<signed char>* known, int cs, int nt, size_t smem, const A& d, int np,
+               cudaStream_t st, bool pdl = false) {
     int dev = 0;
-    cudaGetDevice(&dev);
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) return cudaErrorNotSupported;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(cs, np);
     cfg.blockDim = dim3(nt);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute at[1];
+    cudaLaunchAttribute at[2];
     at[0].id = cudaLaunchAttributeClusterDimension;
     at[0].val.clusterDim.x = cs;
     at[0].val.clusterDim.y = 1;
     at[0].val.clusterDim.z = 1;
+    at[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[1].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    {
-        std::lock_guard<std::mutex> g(mu);
-        const auto key = std::make_pair((const void*)fn, dev);
-        auto it = known.find(key);
-        if (it == known.end()) {
-            int n = 0;
-            bool ok = cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ==
-                          cudaSuccess &&
-                      (cs <= 8 || cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
-                                      cudaSuccess) &&
-                      cudaOccupancyMaxActiveClusters(&n, (const void*)fn, &cfg) == cudaSuccess && n >= 1;
-            if (!ok) cudaGetLastError();
-            it = known.emplace(key, ok).first;
-        }
-        if (!it->second) return cudaErrorNotSupported;
+    if (known[dev] == UNKNOWN) {   // two threads may both ask: the answers agree
+        int n = 0;
+        const bool ok = cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) ==
+                            cudaSuccess &&
+                        (cs <= 8 || cudaFuncSetAttribute((const void*)fn, cudaFuncAttributeNonPortableClusterSizeAllowed,
+                                                         1) == cudaSuccess) &&
+                        cudaOccupancyMaxActiveClusters(&n, (const void*)fn, &cfg) == cudaSuccess && n >= 1;
+        if (!ok) cudaGetLastError();
+        known[dev] = ok ? RUNS : REFUSED;
     }
+    if (known[dev] == REFUSED) return cudaErrorNotSupported;
+    cfg.numAttrs = pdl ? 2 : 1;
     cudaError_t e = cudaLaunchKernelEx(&cfg, fn, d);
     if (e == cudaSuccess) count_launch();
     return e;
 }
 
+#if PFF_RESIDENT == 2
+using Arg = Desc<float>;
+#else
+using Arg = const Desc<float>*;
+#endif
+
 template <int NX, int NY>
-cudaError_t go_size(const Desc<float>* d, int np, cudaStream_t st) {
+cudaError_t go_size(const Arg& d, int np, cudaStream_t st) {
     if constexpr (NX * NY <= RESIDENT_PIXELS) {
+        static std::atomic<signed char> known[MAX_DEVICES];   // per device: can the cluster run
 #if PFF_RESIDENT == 0
         using G = RG<NX, NY, 3>;
-        return go(k_res_mech<NX, NY>, G::CS, G::NT, G::SMEM, d, np, st);
+        return go<Arg>(k_res_mech<NX, NY>, known, G::CS, G::NT, G::SMEM, d, np, st);
+#elif PFF_RESIDENT == 1
+        using G = RG<NX, NY, 1>;
+        return go<Arg>(k_res_bccg<NX, NY>, known, G::CS, G::NT, G::SMEM, d, np, st);
 #else
         using G = RG<NX, NY, 1>;
-        return go(k_res_bccg<NX, NY>, G::CS, G::NT, G::SMEM, d, np, st);
+        return go<Arg>(k_res_lap<NX, NY>, known, G::CS, G::W * 32, G::SMEM, d, np, st, pdl_on());
 #endif
     } else {
         return cudaErrorNotSupported;
@@ -953,7 +1008,7 @@ cudaError_t go_size(const Desc<float>* d, int np, cudaStream_t st) {
 }
 
 template <int NX>
-cudaError_t go_nx(int ny, const Desc<float>* d, int np, cudaStream_t st) {
+cudaError_t go_nx(int ny, const Arg& d, int np, cudaStream_t st) {
     switch (ny) {
         case 16: return go_size<NX, 16>(d, np, st);
         case 32: return go_size<NX, 32>(d, np, st);
@@ -964,7 +1019,7 @@ cudaError_t go_nx(int ny, const Desc<float>* d, int np, cudaStream_t st) {
     }
 }
 
-cudaError_t go_any(int nx, int ny, const Desc<float>* d, int np, cudaStream_t st) {
+cudaError_t go_any(int nx, int ny, const Arg& d, int np, cudaStream_t st) {
     switch (nx) {
         case 16: return go_nx<16>(ny, d, np, st);
         case 32: return go_nx<32>(ny, d, np, st);
@@ -979,10 +1034,14 @@ cudaError_t go_any(int nx, int ny, const Desc<float>* d, int np, cudaStream_t st
 
 #if PFF_RESIDENT == 0
 cudaError_t launch_resident_mech(const Desc<float>* d, int nx, int ny, int np, cudaStream_t st) {
-#else
-cudaError_t launch_resident_bccg(const Desc<float>* d, int nx, int ny, int np, cudaStream_t st) {
-#endif
     return go_any(nx, ny, d, np, st);
 }
+#elif PFF_RESIDENT == 1
+cudaError_t launch_resident_bccg(const Desc<float>* d, int nx, int ny, int np, cudaStream_t st) {
+    return go_any(nx, ny, d, np, st);
+}
+#else
+cudaError_t launch_resident_laplacian(const Desc<float>& d, cudaStream_t st) { return go_any(d.nx, d.ny, d, 1, st); }
+#endif
 
 }  // namespace pff

@@ -30,6 +30,10 @@ cudaError_t launch_mech_cluster(const Desc<float>* d, int np, cudaStream_t st);
 constexpr int RESIDENT_PIXELS = 1 << 14;
 cudaError_t launch_resident_mech(const Desc<float>* d, int nx, int ny, int np, cudaStream_t st);
 cudaError_t launch_resident_bccg(const Desc<float>* d, int nx, int ny, int np, cudaStream_t st);
+// the Laplacian of one small FP32 field (d.r[0] -> d.q[0], d.tw, sizes and mode constants) in one launch;
+// both fields on 8-byte boundaries (a lane moves two adjacent pixels)
+cudaError_t launch_resident_laplacian(const Desc<float>& d, cudaStream_t st);
+inline bool resident_aligned(const void* a, const void* b) { return (((size_t)a | (size_t)b) & 7) == 0; }
 void launch_convert_d2f(float* dst, const double* src, size_t n, cudaStream_t st);
 void launch_convert_f2d(double* dst, const float* src, size_t n, cudaStream_t st);
 

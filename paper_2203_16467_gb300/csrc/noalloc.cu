@@ -27,19 +27,15 @@ constexpr int NA_TW = 2 * NA_MAX;   // twiddle tables for lengths up to NA_MAX
 
 static __device__ __align__(256) double2 g_na_spectrum[(size_t)NA_MAX * NA_WP];
 static __device__ __align__(256) double2 g_na_twiddles[NA_TW];
-static __device__ __align__(256) Desc<double> g_na_desc;
 static __device__ __align__(256) float2 g_na_spectrum_f[(size_t)NA_MAX * NA_WP];
 static __device__ __align__(256) float2 g_na_twiddles_f[NA_TW];
-static __device__ __align__(256) Desc<float> g_na_desc_f;
 
 struct DeviceSymbols {
     bool ready = false;
     double2* spectrum = nullptr;
     double2* twiddles = nullptr;
-    Desc<double>* desc = nullptr;
     float2* spectrum_f = nullptr;
     float2* twiddles_f = nullptr;
-    Desc<float>* desc_f = nullptr;
 };
 constexpr int NA_MAX_DEVICES = 64;
 DeviceSymbols g_symbols[NA_MAX_DEVICES];
@@ -58,18 +54,16 @@ int setup(int dev, DeviceSymbols& out, const char** msg) {
     std::lock_guard<std::mutex> g(g_mu);
     DeviceSymbols& s = g_symbols[dev];
     if (!s.ready) {
-        void* p[6] = {};
-        if (!symbol(g_na_spectrum, &p[0]) || !symbol(g_na_twiddles, &p[1]) || !symbol(g_na_desc, &p[2]) ||
-            !symbol(g_na_spectrum_f, &p[3]) || !symbol(g_na_twiddles_f, &p[4]) || !symbol(g_na_desc_f, &p[5])) {
+        void* p[4] = {};
+        if (!symbol(g_na_spectrum, &p[0]) || !symbol(g_na_twiddles, &p[1]) || !symbol(g_na_spectrum_f, &p[2]) ||
+            !symbol(g_na_twiddles_f, &p[3])) {
             *msg = "cudaGetSymbolAddress failed";
             return PFF_ERR_CUDA;
         }
         s.spectrum = (double2*)p[0];
         s.twiddles = (double2*)p[1];
-        s.desc = (Desc<double>*)p[2];
-        s.spectrum_f = (float2*)p[3];
-        s.twiddles_f = (float2*)p[4];
-        s.desc_f = (Desc<float>*)p[5];
+        s.spectrum_f = (float2*)p[2];
+        s.twiddles_f = (float2*)p[3];
         static double2 tw[NA_TW];   // host staging without a heap allocation
         static float2 twf[NA_TW];
         tw[0] = make_double2(1.0, 0.0);
@@ -98,9 +92,63 @@ int setup(int dev, DeviceSymbols& out, const char** msg) {
 
 bool pow2_in_range(int n) { return n >= 16 && n <= NA_MAX && (n & (n - 1)) == 0; }
 
-template <typename T, typename C, typename DS>
+// the passes with the descriptor as an argument
+template <typename T, int NX>
+__global__ void __launch_bounds__(RowCfg<T, NX, 1>::NT) k_na_row_fwd(const __grid_constant__ Desc<T> d) {
+    row_fwd_body<T, NX, 1, FCopyIn<T, 1>>(d);
+}
+template <typename T, int NX>
+__global__ void __launch_bounds__(RowCfg<T, NX, 1>::NT) k_na_row_inv(const __grid_constant__ Desc<T> d) {
+    row_inv_body<T, NX, 1, FCopyOut<T, 1>>(d);
+}
+template <typename T, int NY>
+__global__ void __launch_bounds__(ColCfg<T, NY, 1>::NT) k_na_col(const __grid_constant__ Desc<T> d) {
+    col_body<T, NY, 1, FColLapPlain>(d);
+}
+__global__ void __launch_bounds__(64 * COL512_CW) k_na_col512(const __grid_constant__ Desc<float> d) {
+    col512_body<float, 1, FColLapPlain, COL512_CW>(d);
+}
+
+template <typename T>
+void go(void (*fn)(Desc<T>), unsigned blocks, unsigned threads, size_t smem, cudaStream_t st, const Desc<T>& d, int key) {
+    smem_optin((const void*)fn, smem);
+    const bool tm = timing_on();
+    if (tm) timing_begin(key, st);
+    launch_pdl<T>(fn, dim3(blocks), dim3(threads), smem, st, d);
+    if (tm) timing_end(key, st);
+    count_launch();
+}
+template <typename T, int N>
+void rows(bool forward, const Desc<T>& d, cudaStream_t st) {
+    using Cfg = RowCfg<T, N, 1>;
+    go<T>(forward ? k_na_row_fwd<T, N> : k_na_row_inv<T, N>, d.ny / Cfg::ROWS, Cfg::NT, Cfg::SMEM, st, d,
+          forward ? FAM_ROW_FWD * 16 + RF_COPY1 : FAM_ROW_INV * 16 + RI_COPY1);
+}
+template <typename T, int N>
+void columns(const Desc<T>& d, cudaStream_t st) {
+    const int nm = d.nx / 2 + 1, key = FAM_COL * 16 + CO_LAP_PLAIN;
+    if constexpr (N == 512 && sizeof(T) == 4) {
+        using Cfg = Col512Cfg<T, 1, COL512_CW>;
+        go<T>(k_na_col512, (nm + COL512_CW - 1) / COL512_CW, Cfg::NT, Cfg::SMEM, st, d, key);
+    } else {
+        using Cfg = ColCfg<T, N, 1>;
+        go<T>(k_na_col<T, N>, (nm + Cfg::CWE - 1) / Cfg::CWE, Cfg::NT, Cfg::SMEM, st, d, key);
+    }
+}
+#define NA_SIZES(n, CALL)                                  \
+    switch (n) {                                           \
+        case 16: { constexpr int N_ = 16; CALL; } break;   \
+        case 32: { constexpr int N_ = 32; CALL; } break;   \
+        case 64: { constexpr int N_ = 64; CALL; } break;   \
+        case 128: { constexpr int N_ = 128; CALL; } break; \
+        case 256: { constexpr int N_ = 256; CALL; } break; \
+        case 512: { constexpr int N_ = 512; CALL; } break; \
+        default: break;                                    \
+    }
+
+template <typename T, typename C>
 int apply(int nx, int ny, double dx, const T* in_dev, T* out_dev, void* cuda_stream, const char** err_msg,
-          C* spectrum, C* twiddles, Desc<T>* desc_dev, const DS& desc_sym) {
+          C* spectrum, C* twiddles) {
     const char* dummy = nullptr;
     const char** msg = err_msg ? err_msg : &dummy;
     cudaStream_t st = (cudaStream_t)cuda_stream;
@@ -116,15 +164,18 @@ int apply(int nx, int ny, double dx, const T* in_dev, T* out_dev, void* cuda_str
     d.k.inv_n = 1.0 / ((double)nx * (double)ny);
     d.k.two_pi_over_Lx = 2.0 * M_PI / (nx * dx);
     d.k.two_pi_over_Ly = 2.0 * M_PI / (ny * dx);
-    // pageable source: the copy has left d before this call returns
-    if (cudaMemcpyToSymbolAsync(desc_sym, &d, sizeof(d), 0, cudaMemcpyHostToDevice, st) != cudaSuccess) {
-        cudaGetLastError();
-        *msg = "descriptor upload failed";
-        return PFF_ERR_CUDA;
+    bool done = false;
+    if constexpr (sizeof(T) == 4) {
+        if (nx * ny <= RESIDENT_PIXELS && resident_aligned(in_dev, out_dev) && !timing_on()) {
+            done = launch_resident_laplacian(d, st) == cudaSuccess;
+            if (!done) cudaGetLastError();   // no such size or no such cluster here: the three passes
+        }
     }
-    launch_row_fwd<T>(RF_COPY1, nx, ny, desc_dev, 1, st);
-    launch_col<T>(CO_LAP_PLAIN, nx, ny, d.wp, desc_dev, 1, st);
-    launch_row_inv<T>(RI_COPY1, nx, ny, desc_dev, 1, st);
+    if (!done) {
+        NA_SIZES(nx, (rows<T, N_>(true, d, st)));
+        NA_SIZES(ny, (columns<T, N_>(d, st)));
+        NA_SIZES(nx, (rows<T, N_>(false, d, st)));
+    }
     if (take_launch_error() != cudaSuccess) {
         *msg = "kernel launch failed";
         return PFF_ERR_CUDA;
@@ -163,8 +214,7 @@ extern "C" int pff_apply_laplacian_noalloc(int nx, int ny, double dx, const doub
     DeviceSymbols sym;
     int rc = check(nx, ny, dx, in_dev, out_dev, msg, sym);
     if (rc) return rc;
-    return apply<double>(nx, ny, dx, in_dev, out_dev, cuda_stream, msg, sym.spectrum, sym.twiddles, sym.desc,
-                         g_na_desc);
+    return apply<double>(nx, ny, dx, in_dev, out_dev, cuda_stream, msg, sym.spectrum, sym.twiddles);
 }
 
 extern "C" int pff_apply_laplacian_noalloc_f32(int nx, int ny, double dx, const float* in_dev, float* out_dev,
@@ -176,6 +226,5 @@ extern "C" int pff_apply_laplacian_noalloc_f32(int nx, int ny, double dx, const 
     DeviceSymbols sym;
     int rc = check(nx, ny, dx, in_dev, out_dev, msg, sym);
     if (rc) return rc;
-    return apply<float>(nx, ny, dx, in_dev, out_dev, cuda_stream, msg, sym.spectrum_f, sym.twiddles_f,
-                        sym.desc_f, g_na_desc_f);
+    return apply<float>(nx, ny, dx, in_dev, out_dev, cuda_stream, msg, sym.spectrum_f, sym.twiddles_f);
 }
