@@ -73,7 +73,7 @@ __device__ __forceinline__ void dft8(C (&u)[8]) {
 // buf[s*SP + pidx(j)]; p = product of the radices of the previous passes.
 //   butterfly i in [0, M/R): k = i mod p; inputs x[i + r M/R]; twiddle
 //   w^(r k) with w = exp(-+2 pi i/(p R)); outputs y[(i - k) R + k + r p].
-// Twiddles: w^k, w^2k (and w^4k for radix 8) from the table, the rest as products.
+// Twiddles: w^k, w^2k (and w^4k for radix 8) from the table, the rest as products (FP32).
 // TWP: the twiddle table is stored with padded indices (pidx), as when staged in
 // shared memory, so that the strided reads of a warp spread over the banks.
 template <typename T, int M, int R, int G, int NSEQ, int SP, int NT, bool INV, bool TWP = false>
@@ -82,6 +82,9 @@ __device__ __forceinline__ void stockham_pass(typename CT<T>::t* buf, int s0, in
     constexpr int NBS = M / R;           // butterflies per sequence
     constexpr int NB = G * NBS;          // butterflies in the round
     constexpr int PER = (NB + NT - 1) / NT;
+    // FP64: all twiddles from the table (16 of a radix-8 butterfly's 100 FP64 instructions formed the
+    // products; that pipe bounds its passes)
+    constexpr bool TABLE = sizeof(T) == 8;
     C u[PER][8];
 #pragma unroll
     for (int j = 0; j < PER; ++j) {
@@ -108,7 +111,13 @@ __device__ __forceinline__ void stockham_pass(typename CT<T>::t* buf, int s0, in
                 } else {
                     C w2 = tw[TWP ? pidx(2 * idx) : 2 * idx];
                     if (INV) w2.y = -w2.y;
-                    C w3 = cmul(w1, w2);
+                    C w3;
+                    if constexpr (TABLE) {
+                        w3 = tw[TWP ? pidx(3 * idx) : 3 * idx];
+                        if (INV) w3.y = -w3.y;
+                    } else {
+                        w3 = cmul(w1, w2);
+                    }
                     u[j][1] = cmul(u[j][1], w1);
                     u[j][2] = cmul(u[j][2], w2);
                     u[j][3] = cmul(u[j][3], w3);
@@ -116,9 +125,18 @@ __device__ __forceinline__ void stockham_pass(typename CT<T>::t* buf, int s0, in
                         C w4 = tw[TWP ? pidx(4 * idx) : 4 * idx];
                         if (INV) w4.y = -w4.y;
                         u[j][4] = cmul(u[j][4], w4);
-                        u[j][5] = cmul(u[j][5], cmul(w1, w4));
-                        u[j][6] = cmul(u[j][6], cmul(w2, w4));
-                        u[j][7] = cmul(u[j][7], cmul(w3, w4));
+                        if constexpr (TABLE) {
+#pragma unroll
+                            for (int r = 5; r < 8; ++r) {
+                                C w = tw[TWP ? pidx(r * idx) : r * idx];
+                                if (INV) w.y = -w.y;
+                                u[j][r] = cmul(u[j][r], w);
+                            }
+                        } else {
+                            u[j][5] = cmul(u[j][5], cmul(w1, w4));
+                            u[j][6] = cmul(u[j][6], cmul(w2, w4));
+                            u[j][7] = cmul(u[j][7], cmul(w3, w4));
+                        }
                     }
                 }
             }
@@ -188,10 +206,14 @@ __device__ __forceinline__ void cp_async_wait_all() {
 template <typename T, int NX, int NC>
 struct RowCfg {
     static constexpr int M = NX / 2;
-    // rows per block: about 512 complex values per block so that a 512^2 grid
-    // already gives 128+ blocks per component plane
-    static constexpr int ROWS = pow2floor(cmax(1, cmin(16, 512 / (NC * M))));   // divides every ny >= 16
     static constexpr bool F32 = sizeof(T) == 4;
+    // rows per block: about 512 complex values per block so that a 512^2 grid
+    // already gives 128+ blocks per component plane.  FP64 rows of up to 256 points: 256 values, so
+    // that the phases of two or more blocks on an SM overlap (FP64 256^2, us, event-timed: BCCG
+    // iterate 22.1 -> 18.8, direction 13.4 -> 12.6; eight of them 55 -> 49; 512-point rows are
+    // better off with 512: iterate 29.8, with 256 values 31.1)
+    static constexpr int VALUES = !F32 && NX <= 256 ? 256 : 512;
+    static constexpr int ROWS = pow2floor(cmax(1, cmin(16, VALUES / (NC * M))));   // divides every ny >= 16
     // 128 threads for up to 1024 complex values (and the 1536 of an FP32 1024-point three-component
     // row, whose passes then hold seven blocks per SM), else 256
     static constexpr int NT = (NC * ROWS * M >= 1024 && !(F32 && NX == 1024)) ? 256 : 128;
@@ -232,8 +254,12 @@ struct ColCfg {
     static constexpr int CSZ = (int)sizeof(typename CT<T>::t);
     static constexpr int CWMIN = 32 / CSZ;                   // one 32-byte sector per row segment
     // one 32-byte sector per row segment: enough columns per block for full
-    // sectors, and as many blocks as possible
-    static constexpr int CWE = CWMIN;
+    // sectors, and as many blocks as possible.  FP64 columns of 256 points on: one per block, half a
+    // sector (the other half comes from L2 for the next block), since twice the blocks fill the chip
+    // and overlap (us, event-timed, two columns -> one: CG pass 256^2 21.1 -> 14.2, 256 x 512 34.8 -> 24.3,
+    // 512^2 39, 1024^2 135 -> 129, four 512^2 119 -> 108, 2048 x 256 61 -> 54).  Shorter columns keep two
+    // (1024 x 128: 20.7, one column 25.2).
+    static constexpr int CWE = sizeof(T) == 8 && NY >= 256 ? 1 : CWMIN;
     static constexpr int SP = ((padded_len(NY) + 7) / 16) * 16 + 8;   // pitch = 8 (mod 16) slots
     static constexpr int NSEQ = NC * CWE;
     static constexpr int NT = (NSEQ * NY >= 8192) ? 512 : (NSEQ * NY >= 2048 ? 256 : 128);
@@ -948,19 +974,29 @@ __device__ __forceinline__ void gamma_apply(const ModeK<T>& m, int kx, int ky, t
     }
     T qx = T(kx) * m.cx;
     T qy = T(signed_k(ky, m.ny)) * m.cy;
-    T inv;
-    if constexpr (sizeof(T) == 4) inv = rsqrtf(qx * qx + qy * qy);   // 2 ulp, one instruction
-    else inv = T(1) / sqrt(qx * qx + qy * qy);
-    T n1 = qx * inv, n2 = qy * inv;
-    T sc = m.inv_n;
-    C a = v[0], b = v[1], c = v[2];
-    C s1{n1 * a.x + n2 * c.x, n1 * a.y + n2 * c.y};      // zeta n
-    C s2{n1 * c.x + n2 * b.x, n1 * c.y + n2 * b.y};
-    C t{n1 * s1.x + n2 * s2.x, n1 * s1.y + n2 * s2.y};   // n . zeta n
-    T n11 = n1 * n1, n22 = n2 * n2, n12 = n1 * n2;
-    v[0] = C{sc * (T(2) * n1 * s1.x - t.x * n11), sc * (T(2) * n1 * s1.y - t.y * n11)};
-    v[1] = C{sc * (T(2) * n2 * s2.x - t.x * n22), sc * (T(2) * n2 * s2.y - t.y * n22)};
-    v[2] = C{sc * (n1 * s2.x + n2 * s1.x - t.x * n12), sc * (n1 * s2.y + n2 * s1.y - t.y * n12)};
+    if constexpr (sizeof(T) == 8) {
+        // Gamma zeta = zeta - (t . zeta t) t (x) t with t the unit tangent: a division and some 35 FP64
+        // instructions (a root, a division and some 80 in the form below, 40 % of a column pass's FP64 work)
+        const T iq = T(1) / (qx * qx + qy * qy), sc = m.inv_n;
+        const T t11 = qy * qy * iq, t22 = qx * qx * iq, t12 = qx * qy * iq;   // t = n turned by 90 degrees; t12 = -t1 t2
+        const C a = v[0], b = v[1], c = v[2];
+        const C s{sc * (t11 * a.x + t22 * b.x - T(2) * t12 * c.x), sc * (t11 * a.y + t22 * b.y - T(2) * t12 * c.y)};
+        v[0] = C{sc * a.x - t11 * s.x, sc * a.y - t11 * s.y};
+        v[1] = C{sc * b.x - t22 * s.x, sc * b.y - t22 * s.y};
+        v[2] = C{sc * c.x + t12 * s.x, sc * c.y + t12 * s.y};
+    } else {
+        const T inv = rsqrtf(qx * qx + qy * qy);   // 2 ulp, one instruction
+        T n1 = qx * inv, n2 = qy * inv;
+        T sc = m.inv_n;
+        C a = v[0], b = v[1], c = v[2];
+        C s1{n1 * a.x + n2 * c.x, n1 * a.y + n2 * c.y};      // zeta n
+        C s2{n1 * c.x + n2 * b.x, n1 * c.y + n2 * b.y};
+        C t{n1 * s1.x + n2 * s2.x, n1 * s1.y + n2 * s2.y};   // n . zeta n
+        T n11 = n1 * n1, n22 = n2 * n2, n12 = n1 * n2;
+        v[0] = C{sc * (T(2) * n1 * s1.x - t.x * n11), sc * (T(2) * n1 * s1.y - t.y * n11)};
+        v[1] = C{sc * (T(2) * n2 * s2.x - t.x * n22), sc * (T(2) * n2 * s2.y - t.y * n22)};
+        v[2] = C{sc * (n1 * s2.x + n2 * s1.x - t.x * n12), sc * (n1 * s2.y + n2 * s1.y - t.y * n12)};
+    }
 }
 
 // Collocation Laplacian multiplier -|2 pi q|^2 / (nx ny) (Sec. 3.1.2).
