@@ -623,4 +623,61 @@ __device__ __forceinline__ void tangent(int split, T xx, T yy, T xy, T hphi, T l
     }
 }
 
+// FP64: the part of the tangent that depends on the strain, which is fixed while a Newton round's CG runs;
+// its kernels read it (f) instead of the strain.  Spectral: u, w of the frame and g12, with
+// H(e1) = (g12 != 0), H(e2) = (|g12| >= 1) and H(tr) = (sign bit clear): g12 of opposite signs lies in
+// (0, 1) and is kept there (at its ends by an ulp).  Vol.-dev.: f[0] = H(tr).  Isotropic: nothing.
+// A root, two divisions and some 20 further FP64 instructions a pixel less in each CG iteration, whose
+// first pass they bound (us, event-timed: 512^2 58.5 -> 41.4, 256^2 18.6 -> 15.8, 256 x 128 15.6 -> 13.7) for
+// three stores a pixel in each Newton round (512^2 79 -> 101).  FP32 problems form the tangent from the
+// strain each time: a reciprocal root costs them little (2048^2 37.0, from the frame 38.6; 1024^2 15.1
+// and 13.6, whose Newton round loses as much).
+template <typename T> constexpr bool TANGENT_FRAME = sizeof(T) == 8;
+template <typename T>
+__device__ __forceinline__ void tangent_frame(int contact, T xx, T yy, T xy, T (&f)[3]) {
+    if (contact == VOLDEV) {
+        f[0] = hv(xx + yy);
+    } else if (contact == SPECTRAL) {
+        Eig2<T> g(xx, yy, xy);
+        const T above0 = T(1e-300), below1 = T(0.99999999999999989);
+        T m;
+        if (g.deg || !(g.e1 > T(0)) || g.e2 > T(0)) m = hv(g.e1);   // one sign: H(e1) (see tangent)
+        else m = fmin(fmax(g.e1 / (g.e1 - g.e2), above0), below1);
+        f[0] = g.u;
+        f[1] = g.w;
+        f[2] = copysign(m, hv(g.tr) - T(0.5));
+    }
+}
+// C:p from the frame f of the strain (see tangent)
+template <typename T>
+__device__ __forceinline__ void tangent_framed(int contact, const T (&f)[3], T hphi, T lam, T mu, T pxx, T pyy, T pxy,
+                                               T* out) {
+    const T trp = pxx + pyy;
+    if (contact == VOLDEV) {
+        const T K = lam + T(2) * mu / T(3), Ht = f[0];
+        const T q = T(4) / T(9) * trp;
+        out[0] = hphi * (K * Ht * trp + T(2) * mu * (pxx - q)) + K * (T(1) - Ht) * trp;
+        out[1] = hphi * (K * Ht * trp + T(2) * mu * (pyy - q)) + K * (T(1) - Ht) * trp;
+        out[2] = hphi * (T(2) * mu * pxy);
+    } else if (contact == SPECTRAL) {
+        const T u = f[0], w = f[1], g12 = fabs(f[2]);
+        const T P1p = T(0.5) * ((T(1) + u) * pxx + (T(1) - u) * pyy + T(2) * w * pxy);
+        const T P2p = T(0.5) * ((T(1) - u) * pxx + (T(1) + u) * pyy - T(2) * w * pxy);
+        const T Sp = T(0.5) * (-w * pxx + w * pyy + T(2) * u * pxy);
+        const T c1 = g12 > T(0) ? P1p : T(0), c2 = g12 >= T(1) ? P2p : T(0), c3 = g12 * Sp;
+        const T dxx = T(0.5) * (c1 * (T(1) + u) + c2 * (T(1) - u)) - c3 * w;
+        const T dyy = T(0.5) * (c1 * (T(1) - u) + c2 * (T(1) + u)) + c3 * w;
+        const T dxy = T(0.5) * (c1 * w - c2 * w) + c3 * u;
+        const bool open = !signbit(f[2]);
+        const T lp = open ? lam * trp : T(0), lm = open ? T(0) : lam * trp;
+        out[0] = hphi * (lp + T(2) * mu * dxx) + lm + T(2) * mu * (pxx - dxx);
+        out[1] = hphi * (lp + T(2) * mu * dyy) + lm + T(2) * mu * (pyy - dyy);
+        out[2] = hphi * (T(2) * mu * dxy) + T(2) * mu * (pxy - dxy);
+    } else {
+        out[0] = hphi * (lam * trp + T(2) * mu * pxx);
+        out[1] = hphi * (lam * trp + T(2) * mu * pyy);
+        out[2] = hphi * (T(2) * mu * pxy);
+    }
+}
+
 }  // namespace pff

@@ -63,7 +63,7 @@ struct NoCtx {};
 
 // ---------------------------------------------------------------- mechanics
 template <typename T>
-struct FNewtonIn {   // eps* += theta (rounds > 0), sigma(eps_bar + eps*, phi)
+struct FNewtonIn {   // eps* += theta (rounds > 0), sigma(eps_bar + eps*, phi); FP64: the tangent's frame to q
     static constexpr int NR = 0;
     struct Ctx { T eb[3]; int fold; int split; LameC<T> lm; };
     __device__ static bool skip(const Desc<T>& d) { return ldflag(&d.ctrl->nd_a); }
@@ -83,6 +83,13 @@ struct FNewtonIn {   // eps* += theta (rounds > 0), sigma(eps_bar + eps*, phi)
         T lam, mu;
         c.lm.at(d, i, lam, mu);
         stress(c.split, c.eb[0] + e0, c.eb[1] + e1, c.eb[2] + e2, hdeg(d.phi[i]), lam, mu, v);
+        if constexpr (TANGENT_FRAME<T>) {
+            const int contact = contact_of(c.split);
+            T f[3];
+            tangent_frame(contact, c.eb[0] + e0, c.eb[1] + e1, c.eb[2] + e2, f);
+            if (contact == SPECTRAL || contact == VOLDEV) d.q[0][i] = f[0];
+            if (contact == SPECTRAL) { d.q[1][i] = f[1]; d.q[2][i] = f[2]; }
+        }
     }
     __device__ static void finalize(const Desc<T>&, const double*) {}
 };
@@ -159,30 +166,33 @@ struct FNewtonOut {   // R = P sigma; CG start r = p = -R, theta = 0; Newton tes
 template <typename T>
 struct FCgIn {
     static constexpr int NR = 1;
-    struct Ctx { T beta; int upd; int iso; T eb[3]; int split; LameC<T> lm; };
+    struct Ctx { T beta; int upd; int contact; T eb[3]; LameC<T> lm; };
     __device__ static bool skip(const Desc<T>& d) {
         int f = ldflag(&d.ctrl->cg_b);
         if (blockIdx.x == 0 && threadIdx.x == 0) d.ctrl->cg_a = f;
         return f;
     }
     __device__ static Ctx prep(const Desc<T>& d) {
-        Ctx c{T(0), 0, 0, {}, 0, LameC<T>(d)};
+        Ctx c{T(0), 0, contact_of(d.k.split), {}, LameC<T>(d)};
         c.upd = ldflag(&d.ctrl->cg_it) > 0;
         c.beta = T(ldd(&d.ctrl->beta));
-        for (int k = 0; k < 3; ++k) c.eb[k] = T(ldd(&d.ctrl->eps_bar[k]));
-        c.split = d.k.split;
-        c.iso = contact_of(d.k.split) == ISOTROPIC;   // the isotropic tangent does not depend on eps
+        if constexpr (!TANGENT_FRAME<T>)
+            for (int k = 0; k < 3; ++k) c.eb[k] = T(ldd(&d.ctrl->eps_bar[k]));
         return c;
     }
-    // two-phase pixel: all loads of a thread's pixels are issued before any store
-    struct In { T p[3], r[3], e[3], phi, E; };
+    // two-phase pixel: all loads of a thread's pixels are issued before any store.  f: the strain, or the
+    // tangent's frame at it from FNewtonIn (q: idle in the mechanics solve); the isotropic tangent takes neither
+    struct In { T p[3], r[3], f[3], phi, E; };
     __device__ static In load(const Desc<T>& d, const Ctx& c, size_t i) {
         In a;
 #pragma unroll
         for (int k = 0; k < 3; ++k) {
             a.p[k] = d.p[k][i];
             if (c.upd) a.r[k] = d.r[k][i];
-            a.e[k] = c.iso ? T(0) : d.eps[k][i];
+            if constexpr (TANGENT_FRAME<T>)
+                a.f[k] = c.contact == SPECTRAL || (c.contact == VOLDEV && k == 0) ? d.q[k][i] : T(0);
+            else
+                a.f[k] = c.contact == ISOTROPIC ? T(0) : d.eps[k][i];
         }
         a.phi = d.phi[i];
         a.E = d.E[i];
@@ -201,8 +211,11 @@ struct FCgIn {
             for (int k = 0; k < 3; ++k) p[k] = a.p[k];
         }
         T lam = c.lm.lc * a.E, mu = c.lm.mc * a.E;
-        tangent(c.split, c.eb[0] + a.e[0], c.eb[1] + a.e[1], c.eb[2] + a.e[2], hdeg(a.phi), lam, mu,
-                p[0], p[1], p[2], v);
+        if constexpr (TANGENT_FRAME<T>)
+            tangent_framed(c.contact, a.f, hdeg(a.phi), lam, mu, p[0], p[1], p[2], v);
+        else
+            tangent(c.contact, c.eb[0] + a.f[0], c.eb[1] + a.f[1], c.eb[2] + a.f[2], hdeg(a.phi), lam, mu,
+                    p[0], p[1], p[2], v);
         wdot(acc[0], p[0], p[1], p[2], v[0], v[1], v[2]);
     }
     __device__ static void finalize(const Desc<T>& d, const double* tot) {
