@@ -166,18 +166,20 @@ struct FNewtonOut {   // R = P sigma; CG start r = p = -R, theta = 0; Newton tes
 template <typename T>
 struct FCgIn {
     static constexpr int NR = 1;
-    struct Ctx { T beta; int upd; int contact; T eb[3]; LameC<T> lm; };
+    struct Ctx { T beta; int upd; int iso; T eb[3]; int split; LameC<T> lm; };
     __device__ static bool skip(const Desc<T>& d) {
         int f = ldflag(&d.ctrl->cg_b);
         if (blockIdx.x == 0 && threadIdx.x == 0) d.ctrl->cg_a = f;
         return f;
     }
     __device__ static Ctx prep(const Desc<T>& d) {
-        Ctx c{T(0), 0, contact_of(d.k.split), {}, LameC<T>(d)};
+        Ctx c{T(0), 0, 0, {}, 0, LameC<T>(d)};
         c.upd = ldflag(&d.ctrl->cg_it) > 0;
         c.beta = T(ldd(&d.ctrl->beta));
         if constexpr (!TANGENT_FRAME<T>)
             for (int k = 0; k < 3; ++k) c.eb[k] = T(ldd(&d.ctrl->eps_bar[k]));
+        c.split = d.k.split;
+        c.iso = contact_of(d.k.split) == ISOTROPIC;   // the isotropic tangent does not depend on eps
         return c;
     }
     // two-phase pixel: all loads of a thread's pixels are issued before any store.  f: the strain, or the
@@ -190,9 +192,9 @@ struct FCgIn {
             a.p[k] = d.p[k][i];
             if (c.upd) a.r[k] = d.r[k][i];
             if constexpr (TANGENT_FRAME<T>)
-                a.f[k] = c.contact == SPECTRAL || (c.contact == VOLDEV && k == 0) ? d.q[k][i] : T(0);
+                a.f[k] = c.iso || (k > 0 && contact_of(c.split) == VOLDEV) ? T(0) : d.q[k][i];
             else
-                a.f[k] = c.contact == ISOTROPIC ? T(0) : d.eps[k][i];
+                a.f[k] = c.iso ? T(0) : d.eps[k][i];
         }
         a.phi = d.phi[i];
         a.E = d.E[i];
@@ -212,9 +214,9 @@ struct FCgIn {
         }
         T lam = c.lm.lc * a.E, mu = c.lm.mc * a.E;
         if constexpr (TANGENT_FRAME<T>)
-            tangent_framed(c.contact, a.f, hdeg(a.phi), lam, mu, p[0], p[1], p[2], v);
+            tangent_framed(contact_of(c.split), a.f, hdeg(a.phi), lam, mu, p[0], p[1], p[2], v);
         else
-            tangent(c.contact, c.eb[0] + a.f[0], c.eb[1] + a.f[1], c.eb[2] + a.f[2], hdeg(a.phi), lam, mu,
+            tangent(c.split, c.eb[0] + a.f[0], c.eb[1] + a.f[1], c.eb[2] + a.f[2], hdeg(a.phi), lam, mu,
                     p[0], p[1], p[2], v);
         wdot(acc[0], p[0], p[1], p[2], v[0], v[1], v[2]);
     }
