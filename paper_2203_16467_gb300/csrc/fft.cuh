@@ -203,6 +203,12 @@ __device__ __forceinline__ void cp_async_wait_all() {
 
 // ---------------------------------------------------------------------------
 // launch geometry
+// Passes of up to 512 points ask for their half spectra beside the skip test (a skipped launch reads them
+// for nothing): the flag's load and the spectrum's, some 800 cycles each, then overlap.  Solves, ms, after -> beside:
+// phase field 512^2 FP32 3.90 -> 3.79, 256^2 FP64 5.09 -> 5.01; mechanics 256 x 128 FP64 1.87 -> 1.84; eight 512^2
+// problems in streams 14.25 -> 13.94 a load step.  Not FP32 with three components (512^2 mechanics 2.42 -> 2.48).
+template <typename T, int N, int NC> constexpr bool EARLY_SPECTRUM = N <= 512 && (NC == 1 || sizeof(T) == 8);
+
 template <typename T, int NX, int NC>
 struct RowCfg {
     static constexpr int M = NX / 2;
@@ -240,6 +246,7 @@ struct RowCfg {
                                     : NX == 512  ? (NC == 3 ? 9 : 7)
                                     : NX == 256  ? (NC == 3 ? 10 : 6)
                                                  : 1;
+    static constexpr bool EARLY = EARLY_SPECTRUM<T, NX, NC>;   // (inverse passes)
     static constexpr int SP = padded_len(M) + 2;            // pitch (complex): padded M values + slot for k = M
     static constexpr int NSEQ = NC * ROWS;
     // twiddles staged in shared memory: length-M FFT table (padded indices) + the
@@ -427,11 +434,25 @@ __global__ void __launch_bounds__(RowCfg<T, NX, NC>::NT) k_row_fwd_u(const Desc<
     row_fwd_body<T, NX, NC, F>(descs[blockIdx.y]);
 }
 
+// the half-spectrum rows of a row group on their way to shared memory (asynchronous copies)
+template <typename T, int NX, int NC>
+__device__ __forceinline__ void row_inv_stage(const Desc<T>& d, int y0, typename CT<T>::t* buf) {
+    using Cfg = RowCfg<T, NX, NC>;
+    using C = typename CT<T>::t;
+    constexpr int M = Cfg::M, SP = Cfg::SP, ROWS = Cfg::ROWS;
+    const unsigned plane = (unsigned)d.ny * d.wp;   // 32-bit indices: < 2^32 elements
+    for (int t = threadIdx.x; t < Cfg::NSEQ * (M + 1); t += Cfg::NT) {
+        const int s = t / (M + 1), k = t % (M + 1);
+        const int c = s / ROWS, row = s % ROWS;
+        cp_async<sizeof(C)>(&buf[s * SP + pidx(k)], &d.S[c * plane + (unsigned)(y0 + row) * d.wp + k]);
+    }
+}
+
 // Row-inverse pass of one row group y0: a few pixels' epilogue loads are issued
 // first (they land during the staging and the FFT; see PREFETCH), the half-spectrum rows are
-// staged, combined for the complex-to-real transform, transformed back along x,
-// and the epilogue runs on the real values (accumulating F's reductions in acc).
-template <typename T, int NX, int NC, class F>
+// staged (STAGED: already on their way), combined for the complex-to-real transform, transformed back
+// along x, and the epilogue runs on the real values (accumulating F's reductions in acc).
+template <typename T, int NX, int NC, class F, bool STAGED = false>
 __device__ __forceinline__ void row_inv_item(const Desc<T>& d, const typename F::Ctx& ctx, int y0,
                                              typename CT<T>::t* buf, const typename CT<T>::t* tws, Acc<T>* acc) {
     using Cfg = RowCfg<T, NX, NC>;
@@ -450,18 +471,13 @@ __device__ __forceinline__ void row_inv_item(const Desc<T>& d, const typename F:
         }
     }
     const C* twN = tws + Cfg::TWF;
-    const unsigned plane = (unsigned)d.ny * d.wp;   // 32-bit indices: < 2^32 elements
     // complex-to-real pre-processing: Z[k] = A + i B,
     //   A = X[k] + conj(X[M-k]),  B = (X[k] - conj(X[M-k])) e^{+2 pi i k/N}
     // (imaginary parts of X[0] and X[M] are dropped, as for a real inverse); the same two
     // values give Z[M-k] = conj(A) + i conj(B), and Z[M/2] = 2 conj(X[M/2]) (k and M - k
     // together, k < M/2; the k = 0 lane forms Z[0] and Z[M/2]).
-    // stage the half spectrum rows in shared memory (asynchronous copies), then combine
-    for (int t = threadIdx.x; t < Cfg::NSEQ * (M + 1); t += NT) {
-        const int s = t / (M + 1), k = t % (M + 1);
-        const int c = s / ROWS, row = s % ROWS;
-        cp_async<sizeof(C)>(&buf[s * SP + pidx(k)], &d.S[c * plane + (unsigned)(y0 + row) * d.wp + k]);
-    }
+    // stage the half spectrum rows in shared memory, then combine
+    if constexpr (!STAGED) row_inv_stage<T, NX, NC>(d, y0, buf);
     cp_async_wait_all();
     __syncthreads();
     // (a lane's two values replace the two that it read, so the combination runs in place)
@@ -544,12 +560,19 @@ __device__ __forceinline__ void row_inv_body(const Desc<T>& d) {
     C* buf = reinterpret_cast<C*>(smem_raw);
     C* tws = buf + Cfg::NSEQ * Cfg::SP;
     pdl_enter();
+    if constexpr (Cfg::EARLY) {
+        row_inv_stage<T, NX, NC>(d, blockIdx.x * Cfg::ROWS, buf);
+        stage_row_twiddles<T, NX, NC>(d, tws);
+    }
     typename F::Ctx ctx;
-    if (block_prep<F>(d, ctx)) return;
-    stage_row_twiddles<T, NX, NC>(d, tws);
+    if (block_prep<F>(d, ctx)) {
+        if constexpr (Cfg::EARLY) cp_async_wait_all();
+        return;
+    }
+    if constexpr (!Cfg::EARLY) stage_row_twiddles<T, NX, NC>(d, tws);
     constexpr int NRA = F::NR > 0 ? F::NR : 1;
     Acc<T> acc[NRA];
-    row_inv_item<T, NX, NC, F>(d, ctx, blockIdx.x * Cfg::ROWS, buf, tws, &acc[0]);
+    row_inv_item<T, NX, NC, F, Cfg::EARLY>(d, ctx, blockIdx.x * Cfg::ROWS, buf, tws, &acc[0]);
     if constexpr (F::NR > 0) reduce_finalize<F, F::NR, NT>(acc, d, gridDim.x);
 }
 template <typename T, int NX, int NC, class F>
@@ -594,7 +617,9 @@ __device__ __forceinline__ void col_body(const Desc<T>& d) {
     C* buf = reinterpret_cast<C*>(smem_raw);
     pdl_enter();
     ModeK<T> mk;
-    if (block_prep<ColPrep<T, OP>>(d, mk)) return;
+    constexpr bool EARLY = EARLY_SPECTRUM<T, NY, NC>;
+    if constexpr (!EARLY)
+        if (block_prep<ColPrep<T, OP>>(d, mk)) return;
     const C* tw = d.tw + NY;
     if constexpr (Cfg::TW_SMEM) {
         C* tws = buf + Cfg::NSEQ * SP;
@@ -608,6 +633,11 @@ __device__ __forceinline__ void col_body(const Desc<T>& d) {
         const int j = t % CW, ky = (t / CW) % NY, c = t / (CW * NY);
         cp_async<sizeof(C)>(&buf[(c * CW + j) * SP + pidx(ky)], &d.S[c * plane + (unsigned)ky * d.wp + kx0 + j]);
     }
+    if constexpr (EARLY)
+        if (block_prep<ColPrep<T, OP>>(d, mk)) {
+            cp_async_wait_all();
+            return;
+        }
     cp_async_wait_all();
     __syncthreads();
     fft_smem<T, NY, Cfg::NSEQ, SP, NT, false, Cfg::TW_SMEM>(buf, tw);
@@ -726,18 +756,24 @@ __device__ __forceinline__ void stage_col512_twiddles(const Desc<T>& d, typename
 }
 
 // Column pass of the CW columns kx0.. of the half spectrum (64 CW threads).
-template <typename T, int NC, class OP, int CW>
-__device__ __forceinline__ void col512_item(const Desc<T>& d, const ModeK<T>& mk, int kx0, typename CT<T>::t* xb,
-                                            const typename CT<T>::t* tws, Acc<T>* acc = nullptr) {
-    using C = typename CT<T>::t;
-    const int j = threadIdx.x % CW, t = threadIdx.x / CW;
-    const int kx = kx0 + j;
+template <typename T, int NC, int CW>
+__device__ __forceinline__ void col512_load(const Desc<T>& d, int kx0, typename CT<T>::t (&u)[NC][8]) {
+    const int t = threadIdx.x / CW, kx = kx0 + threadIdx.x % CW;
     const unsigned plane = (unsigned)d.ny * d.wp;   // 32-bit indices: < 2^32 elements
-    C u[NC][8];
 #pragma unroll
     for (int c = 0; c < NC; ++c)
 #pragma unroll
         for (int m = 0; m < 8; ++m) u[c][m] = d.S[c * plane + (unsigned)(t + 64 * m) * d.wp + kx];
+}
+// (u: the columns, from col512_load)
+template <typename T, int NC, class OP, int CW>
+__device__ __forceinline__ void col512_item(const Desc<T>& d, const ModeK<T>& mk, int kx0, typename CT<T>::t* xb,
+                                            const typename CT<T>::t* tws, typename CT<T>::t (&u)[NC][8],
+                                            Acc<T>* acc = nullptr) {
+    using C = typename CT<T>::t;
+    const int j = threadIdx.x % CW, t = threadIdx.x / CW;
+    const int kx = kx0 + j;
+    const unsigned plane = (unsigned)d.ny * d.wp;
     cp_async_wait_all();   // staged twiddles (a no-op when the caller has waited already)
     __syncthreads();
     fft512_reg<T, false, NC, CW>(u, t, t, xb + j * COL512_XS, tws);
@@ -768,11 +804,23 @@ __device__ __forceinline__ void col512_body(const Desc<T>& d) {
     C* xb = tws + padded_len(512);
     pdl_enter();
     ModeK<T> mk;
-    if (block_prep<ColPrep<T, OP>>(d, mk)) return;
-    stage_col512_twiddles<T>(d, tws);   // waited for inside the item, after its loads are issued
+    C u[NC][8];
+    constexpr bool EARLY = EARLY_SPECTRUM<T, 512, NC>;
+    if constexpr (EARLY) {
+        stage_col512_twiddles<T>(d, tws);   // waited for inside the item
+        col512_load<T, NC, CW>(d, blockIdx.x * CW, u);
+    }
+    if (block_prep<ColPrep<T, OP>>(d, mk)) {
+        if constexpr (EARLY) cp_async_wait_all();
+        return;
+    }
+    if constexpr (!EARLY) {
+        stage_col512_twiddles<T>(d, tws);
+        col512_load<T, NC, CW>(d, blockIdx.x * CW, u);
+    }
     constexpr int NRA = ColNR<OP>::value > 0 ? ColNR<OP>::value : 1;
     Acc<T> acc[NRA];
-    col512_item<T, NC, OP, CW>(d, mk, blockIdx.x * CW, xb, tws, acc);
+    col512_item<T, NC, OP, CW>(d, mk, blockIdx.x * CW, xb, tws, u, acc);
     if constexpr (ColNR<OP>::value > 0) reduce_finalize<OP, ColNR<OP>::value, 64 * CW>(acc, d, gridDim.x);
 }
 template <typename T, int NC, class OP, int CW = COL512_CW>

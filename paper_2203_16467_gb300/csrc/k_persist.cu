@@ -170,7 +170,9 @@ __device__ __noinline__ bool col_phase(const Desc<float>& d, float2* work, const
     const ModeK<float> mk(d);
     for (int item = blockIdx.x; item < (d.nx / 2 + PB_CW) / PB_CW; item += gridDim.x) {   // mode columns only
         __syncthreads();
-        col512_item<float, 1, OP, PB_CW>(d, mk, item * PB_CW, work, ctw);
+        float2 u[1][8];
+        col512_load<float, 1, PB_CW>(d, item * PB_CW, u);
+        col512_item<float, 1, OP, PB_CW>(d, mk, item * PB_CW, work, ctw, u);
     }
     DF none[1];
     return grid_sync<0>(d.ctrl, d.part, none, NoFin{}, spin);
