@@ -32,10 +32,17 @@
 // evaluated explicitly).
 //
 // Order of the exchanges.  A CTA sends into a buffer of another only after that one has read the
-// buffer's previous contents: it has, before, received the sums (slot 1) to which the other
-// contributed after that read; and a receiver arms an mbarrier's phase when it waits for it, so that
+// buffer's previous contents; and a receiver arms an mbarrier's phase when it waits for it, so that
 // bytes that arrive earlier already count for the phase they belong to (the previous one has completed).
-// Sums use two slots in turn, each with its own mbarrier, for the same reason.  Every CTA sums the
+//   modes, rows: a CTA that has all its rows knows that every CTA has read its modes (the rows are
+//     made of them) and its previous rows (a CTA sends its modes after reading those);
+//   sums, slot 0 (p.Ap, p.Jp): sent beside an operator, when all that a CTA knows of the others are the
+//     sums it has received; those before it were slot 1's, and each CTA contributed to them after reading
+//     slot 0.  The wait for the modes would not do: a CTA without mode columns (1 to 7 of each cluster)
+//     waits for none;
+//   sums, slot 1 (everything else): sent after an operator, of which each CTA has received all rows,
+//     which every CTA made possible after reading slot 1.
+// (tests/test_resident_exchanges.py plays this order with late CTAs.)  Every CTA sums the
 // same partials in the same order, so all take the same decisions.  Waits are bounded (about two
 // seconds, then status bit 8); the cluster barriers at the start and the end are reached by every
 // thread once.
@@ -839,10 +846,10 @@ __global__ void __launch_bounds__(RG<NX, NY, 1>::NT, 1) k_res_bccg(const Desc<fl
             for (int k = 0; k < 7; ++k) sh[k * W * 32 + threadIdx.x] = t.on ? acc[k].df() : DF{0.f, 0.f};
         }
         __syncthreads();
-        many_sums<7, W, CS>(s, sh, 0, t.rank, t.warp, t.lane);
+        many_sums<7, W, CS>(s, sh, 1, t.rank, t.warp, t.lane);
         if (scalar) {
-            x8 = take_many<7, CS>(s, 0, p0, t.lane);
-            p0 ^= 1u;
+            x8 = take_many<7, CS>(s, 1, p1, t.lane);
+            p1 ^= 1u;
             rr = __shfl_sync(FULLW, x8, 0);
             beta = (rr - __shfl_sync(FULLW, x8, 4)) * irp;
             ++it;
