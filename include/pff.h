@@ -166,7 +166,7 @@ typedef struct pff_step_report {
     int n_active;
     int istar;                 /* linear index of argmax -F_phi */
     int broken;                /* C_bar < C_broken */
-    int status;                /* PFF_OK or PFF_ERR_NOT_CONVERGED */
+    int status;                /* PFF_OK, PFF_ERR_NOT_CONVERGED or PFF_ERR_BARRIER_TIMEOUT */
     int bccg_clamp_iters;      /* BCCG iterations in which the projection onto v >= v_con changed v */
     double dt;                 /* time-dependent method: the time step for the next step (units of eta/(G_c/ell)) */
     int inner_iters;           /* alternating minimisation: inner iterations; time-dependent: phase-field tries */
@@ -450,13 +450,17 @@ int pff_set_persistent(int on);
  * counterpart in the paper. */
 int pff_set_cluster_mechanics(int on);
 
-/* Wait limit of every grid barrier of the persistent solve, in SM clock cycles
+/* Wait limit of every grid barrier of the persistent solve and of every exchange
+ * of the one-launch solves of small FP32 grids, in SM clock cycles
  * (cycles > 0; 0 restores the default of 4e9 cycles, about two seconds at the
- * maximum clock).  A block that is not released within the limit sets the
- * problem's abort flag and returns; the other blocks return at their next
- * barrier, the solve ends with PFF_ERR_BARRIER_TIMEOUT, the phase field is left
- * unchanged and the handle stays usable.  A short limit (one cycle) makes the
- * first barrier time out, which tests use to exercise that path.  Takes effect
+ * maximum clock).  A block that is not released within the limit gives the solve
+ * up, and with it the other blocks.  The call ends with PFF_ERR_BARRIER_TIMEOUT
+ * (pff_step_load and pff_batch_step stop there; in a batch the problem's report
+ * has that status and nothing else, the other problems' step counts), the phase
+ * field, and eps* after a mechanics solve, are as before the solve and the handle
+ * stays usable; pff_apply_laplacian_noalloc_f32, which cannot report it, leaves
+ * NaN.  A short limit (one cycle) makes the first wait run out, which tests use
+ * to exercise that path.  Takes effect
  * at the next launch.  Negative values: PFF_ERR_INVALID_ARG.  No counterpart in
  * the paper. */
 int pff_set_barrier_spin_limit(long long cycles);

@@ -750,7 +750,7 @@ static int mech_solve_group(Group& g, int max_cg, int max_newton, pff_problem* e
     const int nx = g.nx, ny = g.ny, wp = g.wp, np = g.np;
     cudaStream_t st = g.st;
     int rc;
-    if (resident_solve<T>(0, g)) return 0;   // folds the last update itself
+    if (resident_solve<T>(0, g)) return 0;   // folds the last update itself (status bit 8: given up)
     if (mech_cluster_group<T>(g)) return 0;
     for (int round = 0; round <= max_newton; ++round) {
         launch_row_fwd<T>(RF_NEWTON, nx, ny, d, np, st);
@@ -857,6 +857,11 @@ static void fill_report(const Ctrl& c, int split, pff_step_report* r) {
     r->status = (c.status & 8) ? PFF_ERR_BARRIER_TIMEOUT : c.status ? PFF_ERR_NOT_CONVERGED : PFF_OK;
 }
 
+// A solve that was given up because a wait ran out (its result is not applied).
+static int timed_out(pff_problem* h) {
+    return fail(h, PFF_ERR_BARRIER_TIMEOUT, "a sub-problem solve's wait between its thread blocks timed out");
+}
+
 static Group single_group(pff_problem* h) {
     Group g;
     g.nx = h->nx; g.ny = h->ny; g.wp = h->wp; g.prec = h->prec; g.np = 1;
@@ -940,6 +945,7 @@ static int am_increment(pff_problem* h, pff_step_report* out) {
         if ((rc = pf_solve_group<T>(g, p.pf_max_iter, h, warmed))) break;
         if ((rc = poll<T>(g, true, h))) break;
         const Ctrl& c = g.h_ctrl[0];
+        if (c.status & 8) { rc = timed_out(h); break; }
         dphi = c.dphi;
         cg += c.cg_total;
         pf += c.pf_it;
@@ -976,18 +982,23 @@ static int td_step(pff_problem* h, pff_step_report* out) {
     if (h->td_dt <= 0.0) h->td_dt = p.dt_max;
     double dt = h->td_dt;
     bool warmed = h->graphs.exec[0] || h->graphs.exec[1];
+    auto give_up = [&](int code) {   // the method's control values do not outlive it
+        set_method_ctrl(h, 0, 0.0, 0, 0);
+        return code;
+    };
     if ((rc = set_method_ctrl(h, 1, p.Gc / p.ell / dt, 0, 1))) return rc;
     launch_step_begin<T>(d, 1, h->st);
-    if ((rc = mech_solve_group<T>(g, p.mech_max_cg, p.mech_max_newton, h, warmed))) return rc;
+    if ((rc = mech_solve_group<T>(g, p.mech_max_cg, p.mech_max_newton, h, warmed))) return give_up(rc);
     lap_phi_group<T>(g, false);
     launch_elem<T>(EL_SAVE_PHI, h->nx, h->ny, d, 1, h->st);
     int tries = 0, pf = 0, clamps = 0, fulls = 0, status = 0;
     double dphi = 0.0;
     for (;;) {
-        if (tries > 0 && (rc = set_method_ctrl(h, 1, p.Gc / p.ell / dt, 0, 1))) return rc;
-        if ((rc = pf_solve_group<T>(g, p.pf_max_iter, h, warmed))) return rc;
-        if ((rc = poll<T>(g, true, h))) return rc;
+        if (tries > 0 && (rc = set_method_ctrl(h, 1, p.Gc / p.ell / dt, 0, 1))) return give_up(rc);
+        if ((rc = pf_solve_group<T>(g, p.pf_max_iter, h, warmed))) return give_up(rc);
+        if ((rc = poll<T>(g, true, h))) return give_up(rc);
         const Ctrl& c = g.h_ctrl[0];
+        if (c.status & 8) return give_up(timed_out(h));
         dphi = c.dphi;
         pf += c.pf_it;
         clamps += c.pf_clamp_iters;
@@ -1432,6 +1443,7 @@ int pff_step_load(pff_problem* h, int n_steps, pff_step_report* out, int* steps_
         int rc = run_group_step(g, h->prm, h->prm.compute_energies != 0, h);
         if (rc) return rc;
         const Ctrl& c = g.h_ctrl[0];
+        if (c.status & 8) return timed_out(h);
         if (out) fill_report(c, h->split, &out[s]);
         if (c.status) status = PFF_ERR_NOT_CONVERGED;
         if (steps_done) *steps_done = s + 1;
@@ -1467,6 +1479,7 @@ int pff_solve_mechanics(pff_problem* h, pff_step_report* out) {
     };
     rc = h->prec == PFF_FP64 ? body(double()) : body(float());
     if (rc) return rc;
+    if (g.h_ctrl[0].status & 8) return timed_out(h);
     if (out) {
         std::memset(out, 0, sizeof(*out));
         fill_report(g.h_ctrl[0], h->split, out);
@@ -1521,6 +1534,7 @@ int pff_solve_phase_field(pff_problem* h, pff_step_report* out) {
     int rc = h->prec == PFF_FP64 ? body(double()) : body(float());
     if (rc) return rc;
     const Ctrl& c = g.h_ctrl[0];
+    if (c.status & 8) return timed_out(h);
     if (out) {
         std::memset(out, 0, sizeof(*out));
         fill_report(c, h->split, out);
@@ -1827,7 +1841,8 @@ int pff_batch_step(pff_batch* b, int n_steps, pff_step_report* reports, int* ste
     if (steps_done)
         for (int i = 0; i < b->max_slots; ++i) steps_done[i] = 0;
     int status = PFF_OK;
-    for (int s = 0; s < n_steps; ++s) {
+    pff_problem* late = nullptr;   // a problem whose step was given up
+    for (int s = 0; s < n_steps && !late; ++s) {
         int rc = build_groups(b);
         if (rc) return rc;
         if (b->groups.empty()) break;
@@ -1875,12 +1890,25 @@ int pff_batch_step(pff_batch* b, int n_steps, pff_step_report* reports, int* ste
             for (size_t j = 0; j < bg.slots.size(); ++j) {
                 int i = bg.slots[j];
                 const Ctrl& c = bg.h_ctrl[j];
+                if (c.status & 8) {   // not a step: nothing of it but the status is reported
+                    late = b->slot[i];
+                    if (reports) {
+                        std::memset(&reports[(size_t)i * n_steps + s], 0, sizeof(*reports));
+                        reports[(size_t)i * n_steps + s].status = PFF_ERR_BARRIER_TIMEOUT;
+                    }
+                    continue;
+                }
                 if (reports) fill_report(c, b->slot[i]->split, &reports[(size_t)i * n_steps + s]);
                 if (steps_done) steps_done[i] = s + 1;
                 if (c.status) status = PFF_ERR_NOT_CONVERGED;
                 if (c.broken) b->slot[i]->broken = true;
             }
         }
+    }
+    if (late) {
+        const int rc = timed_out(late);
+        b->err = late->err;
+        return rc;
     }
     return status;
 }

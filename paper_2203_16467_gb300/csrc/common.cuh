@@ -68,7 +68,7 @@ struct Ctrl {
     // post-step (Algorithm 4 lines 12-14)
     double rep_eps_bar[3], sig_bar[3], C_bar, dphi, Fe, Ff;
     int incremented, broken;
-    int status;             // bit0: mechanics cap hit, bit1: BCCG cap hit
+    int status;             // bit0: mechanics cap hit, bit1: BCCG cap hit, bit3: a wait ran out
     unsigned counter;       // last-block reduction counter (reset by the last block)
     // set by the host for the alternating-minimisation / time-dependent methods
     double eta_dt_override; // eta/dt of the phase-field step when use_override

@@ -252,15 +252,19 @@ int persist_bccg_blocks(int share_den) {
     return b;
 }
 
-// Wait limit of the grid barriers in clock cycles (0: the default of about two seconds).
+// Wait limit of the grid barriers and of the resident solves' exchanges in clock cycles (0: the default
+// of about two seconds).
 static std::atomic<long long> g_spin{0};
 void persist_set_spin(long long cycles) { g_spin.store(cycles > 0 ? cycles : 0); }
+long long barrier_spin_limit() {
+    const long long spin = g_spin.load();
+    return spin > 0 ? spin : PB_SPIN_CYCLES;
+}
 
 // Launches the persistent solve of one FP32 512 x 512 problem (after its BCCG start).
 cudaError_t launch_persist_bccg(const Desc<float>* d, int max_iters, int blocks, cudaStream_t st) {
     if (blocks < 1) return cudaErrorInvalidConfiguration;
-    long long spin = g_spin.load();
-    if (spin <= 0) spin = PB_SPIN_CYCLES;
+    long long spin = barrier_spin_limit();
     void* args[] = {(void*)&d, (void*)&max_iters, (void*)&spin};
     cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_bccg512, dim3(blocks), dim3(PB_NT), args, PB_SMEM, st);
     count_launch();

@@ -43,9 +43,15 @@
 //   sums, slot 1 (everything else): sent after an operator, of which each CTA has received all rows,
 //     which every CTA made possible after reading slot 1.
 // (tests/test_resident_exchanges.py plays this order with late CTAs.)  Every CTA sums the
-// same partials in the same order, so all take the same decisions.  Waits are bounded (about two
-// seconds, then status bit 8); the cluster barriers at the start and the end are reached by every
-// thread once.
+// same partials in the same order, so all take the same decisions.
+//
+// Waits are bounded (pff_set_barrier_spin_limit; about two seconds by default).  A CTA whose wait ran
+// out goes on to the next block barrier that asks for it (the answer is the barrier's, so all its warps
+// leave together), stops sending, and so makes the others' waits run out; a CTA that was sent partial
+// results meanwhile learns of it at the end (leave).  Nothing of a solve is stored before that: eps*, v
+// and the control block stay as they were, status bit 8 is set, and the kernels that follow in a load
+// step leave the state alone.  The cluster barriers at the start and the end are reached by every thread
+// once.
 //
 // Arithmetic: the pixel functions, mode multipliers and finalizers of the per-kernel path; a
 // private copy of the control block in each CTA's shared memory takes the finalizers' results and
@@ -61,7 +67,6 @@ namespace {
 
 using C = float2;
 constexpr int MAXR = 8;                             // values of a reduction
-constexpr long long SPIN_CYCLES = 4000000000LL;     // wait limit (about two seconds)
 constexpr unsigned FULLW = 0xffffffffu;
 
 // ---------------------------------------------------------------- cluster primitives
@@ -88,6 +93,16 @@ __device__ __forceinline__ void bar_init(unsigned bar) {
 __device__ __forceinline__ void bar_arm(unsigned bar, unsigned bytes) {
     asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(bar), "r"(bytes) : "memory");
 }
+// has the phase completed: now, and waiting a little for it
+__device__ __forceinline__ bool bar_test(unsigned bar, unsigned parity) {
+    unsigned ok;
+    asm volatile(
+        "{\n.reg .pred p;\nmbarrier.test_wait.parity.acquire.cluster.shared::cta.b64 p, [%1], %2;\nselp.u32 %0, 1, 0, p;\n}"
+        : "=r"(ok)
+        : "r"(bar), "r"(parity)
+        : "memory");
+    return ok != 0;
+}
 __device__ __forceinline__ bool bar_try(unsigned bar, unsigned parity) {
     unsigned ok;
     asm volatile(
@@ -96,6 +111,10 @@ __device__ __forceinline__ bool bar_try(unsigned bar, unsigned parity) {
         : "r"(bar), "r"(parity)
         : "memory");
     return ok != 0;
+}
+// a plain store to the shared memory of a CTA of the cluster
+__device__ __forceinline__ void put(unsigned a, int v) {
+    asm volatile("st.shared::cluster.u32 [%0], %1;" ::"r"(a), "r"(v) : "memory");
 }
 __device__ __forceinline__ unsigned cta_rank() {
     unsigned r;
@@ -134,20 +153,24 @@ struct Shared {              // per-CTA scalars
     unsigned long long bar[4];   // mbarriers: modes, rows, sums slot 0, sums slot 1
     Ctrl ctrl;
     Desc<float> d;           // the problem's descriptor with ctrl pointing here
-    volatile int dead;       // a wait ran out
+    long long spin;          // wait limit in clock cycles
+    volatile int dead;       // a wait of this CTA ran out
+    volatile int any;        // a wait of some CTA ran out (written before the last cluster barrier)
 };
 enum { B_MODES = 0, B_ROWS = 1, B_SUM0 = 2, B_SUM1 = 3 };
 
-// Wait for `parity` of an mbarrier; every lane polls, at most SPIN_CYCLES (then s.dead).
+// Wait for `parity` of an mbarrier; every lane polls, at most s.spin cycles (then s.dead).
 __device__ __forceinline__ void await(Shared& s, int which, unsigned parity) {
     const unsigned bar = s32(&s.bar[which]);
-    if (bar_try(bar, parity)) return;
+    if (bar_test(bar, parity)) return;
     const long long t0 = clock64();
     while (!s.dead) {
-        if (bar_try(bar, parity)) return;
-        if (clock64() - t0 > SPIN_CYCLES) s.dead = 1;
+        if (clock64() - t0 > s.spin) s.dead = 1;
+        else if (bar_try(bar, parity)) return;
     }
 }
+// A block barrier: has a wait of this CTA run out (the same answer in every thread)?
+__device__ __forceinline__ bool sync_dead(const Shared& s) { return __syncthreads_or(s.dead) != 0; }
 
 // ---------------------------------------------------------------- FFTs within a warp
 // Stage twiddles of the lane FFT: w[i] for the half-width h = 16 >> i: exp(-pi i (lane mod h) / h) in
@@ -461,9 +484,16 @@ __device__ __forceinline__ void scalar_arrive() { asm volatile("bar.arrive 1, %0
 template <int NT>
 __device__ __forceinline__ void scalar_join() { asm volatile("bar.sync 1, %0;" ::"n"(NT) : "memory"); }
 
+__device__ __forceinline__ void init(Shared& s, long long spin) {   // one thread, before the cluster's start
+    s.spin = spin;
+    s.dead = 0;
+    s.any = 0;
+    for (int b = 0; b < 4; ++b) bar_init(s32(&s.bar[b]));
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+}
 // Control block, descriptor, column twiddles; mbarriers; then the cluster's start.
 template <class G, int NY>
-__device__ __forceinline__ void stage(const Desc<float>& d, Shared& s, C* sm) {
+__device__ __forceinline__ void stage(const Desc<float>& d, Shared& s, C* sm, long long spin) {
     const int* src = reinterpret_cast<const int*>(d.ctrl);
     int* dst = reinterpret_cast<int*>(&s.ctrl);
     for (int i = threadIdx.x; i < (int)(sizeof(Ctrl) / 4); i += G::NT) dst[i] = __ldcg(src + i);
@@ -471,38 +501,43 @@ __device__ __forceinline__ void stage(const Desc<float>& d, Shared& s, C* sm) {
     int* dd = reinterpret_cast<int*>(&s.d);
     for (int i = threadIdx.x; i < (int)(sizeof(Desc<float>) / 4); i += G::NT) dd[i] = sd[i];
     for (int i = threadIdx.x; i < NY; i += G::NT) sm[G::O_TWC + i] = d.tw[NY + i];
-    if (threadIdx.x == 0) {
-        s.dead = 0;
-        for (int b = 0; b < 4; ++b) bar_init(s32(&s.bar[b]));
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
+    if (threadIdx.x == 0) init(s, spin);
     __syncthreads();
     if (threadIdx.x == 0) s.d.ctrl = &s.ctrl;
     __syncthreads();
     cluster_sync_all();
 }
 
-// Control block back (rank 0) and the cluster's end; a CTA whose wait ran out gives what may still be
-// on its way to it time to arrive.
+// The cluster's end: true when no wait of any CTA ran out.  Otherwise what is still on its way to a CTA
+// gets time to arrive before that one exits.
+template <int CS>
+__device__ __forceinline__ bool finished(Shared& s) {
+    __syncthreads();   // no wait of this CTA from here on
+    if (s.dead && threadIdx.x < CS) put(at_rank(s32((const void*)&s.any), threadIdx.x), 1);
+    cluster_sync_all();
+    if (!s.any) return true;
+    const long long t0 = clock64();
+    while (clock64() - t0 < 1000000) {}
+    return false;
+}
+// ... and the control block back (rank 0), or status bit 8 alone.
 template <class G>
-__device__ __forceinline__ void leave(const Desc<float>& d, Shared& s, unsigned rank) {
-    __syncthreads();
+__device__ __forceinline__ bool leave(const Desc<float>& d, Shared& s, unsigned rank) {
+    if (!finished<G::CS>(s)) {
+        if (rank == 0 && threadIdx.x == 0) atomicOr(&d.ctrl->status, 8);
+        return false;
+    }
     if (rank == 0) {
         const int* src = reinterpret_cast<const int*>(&s.ctrl);
         int* dst = reinterpret_cast<int*>(d.ctrl);
         for (int i = threadIdx.x; i < (int)(sizeof(Ctrl) / 4); i += G::NT) dst[i] = src[i];
     }
-    if (s.dead) {
-        const long long t0 = clock64();
-        while (clock64() - t0 < 1000000) {}
-    }
-    cluster_sync_all();
-    if (s.dead && threadIdx.x == 0) atomicOr(&d.ctrl->status, 8);
+    return true;
 }
 
 // ---------------------------------------------------------------- mechanics (Sec. 3.1.1)
 template <int NX, int NY>
-__global__ void __launch_bounds__(RG<NX, NY, 3>::NT, 1) k_res_mech(const Desc<float>* __restrict__ descs) {
+__global__ void __launch_bounds__(RG<NX, NY, 3>::NT, 1) k_res_mech(const Desc<float>* __restrict__ descs, long long spin) {
     using G = RG<NX, NY, 3>;
     constexpr int E = G::ER, PP = 2 * E, NT = G::NT, CS = G::CS, W = G::W;
     const Desc<float>& d = descs[blockIdx.y];
@@ -510,7 +545,7 @@ __global__ void __launch_bounds__(RG<NX, NY, 3>::NT, 1) k_res_mech(const Desc<fl
     __shared__ Shared s;
     __shared__ DF sh[W * 32];
     C* sm = reinterpret_cast<C*>(smem_raw);
-    stage<G, NY>(d, s, sm);
+    stage<G, NY>(d, s, sm, spin);
     Lane<G> t;
     lane_setup<NX, NY, 3>(t, d, s, sm);
     const ModeK<float> mk(s.d);
@@ -545,18 +580,13 @@ __global__ void __launch_bounds__(RG<NX, NY, 3>::NT, 1) k_res_mech(const Desc<fl
         target2 = target * target;
     }
     C z[3 * E];
-    for (int round = 0;; ++round) {          // Newton rounds
-        const bool fold = round > 0;
-        if (fold && t.on) {
+    bool fold = false, dead = false;
+    for (;; fold = true) {                   // Newton rounds
+        if (fold) {
 #pragma unroll
-            for (int q = 0; q < PP; ++q) {
-                const unsigned i = pix + (q >> 1) * 2 * G::LR + (q & 1);
+            for (int q = 0; q < PP; ++q)
 #pragma unroll
-                for (int k = 0; k < 3; ++k) {
-                    ep[q][k] += th[q][k];
-                    d.eps[k][i] = ep[q][k];
-                }
-            }
+                for (int k = 0; k < 3; ++k) ep[q][k] += th[q][k];
         }
         if (fold && linear) break;   // a linear model takes one Newton step: folded, done
         if (!scalar) {
@@ -600,8 +630,8 @@ __global__ void __launch_bounds__(RG<NX, NY, 3>::NT, 1) k_res_mech(const Desc<fl
             }
             if (t.lane == 0) s.stop = stop;
         }
-        __syncthreads();
-        if (s.stop || s.dead) break;   // Newton stopping test (or the round limit)
+        dead = sync_dead(s);
+        if (s.stop || dead) break;     // Newton stopping test (or the round limit)
         bool first = true;
         do {                                // CG iterations
             if (!scalar) {
@@ -636,8 +666,8 @@ __global__ void __launch_bounds__(RG<NX, NY, 3>::NT, 1) k_res_mech(const Desc<fl
                 }
             }
             first = false;
-            __syncthreads();
-            if (s.stop || s.dead) break;    // p.Ap <= 0: no update
+            dead = sync_dead(s);
+            if (s.stop || dead) break;      // p.Ap <= 0: no update
             if (!scalar) {
                 const float alpha = s.alpha;
                 Acc<float> acc;
@@ -666,9 +696,9 @@ __global__ void __launch_bounds__(RG<NX, NY, 3>::NT, 1) k_res_mech(const Desc<fl
                     s.stop = stop;
                 }
             }
-            __syncthreads();
-        } while (!s.stop && !s.dead);
-        if (s.dead) break;
+            dead = sync_dead(s);
+        } while (!s.stop && !dead);
+        if (dead) break;
     }
     __syncthreads();
     if (scalar && t.lane == 0) {    // results, and the flags as the per-kernel path leaves them
@@ -683,13 +713,20 @@ __global__ void __launch_bounds__(RG<NX, NY, 3>::NT, 1) k_res_mech(const Desc<fl
         c.nd_a = c.nd_b = c.cg_a = c.cg_b = 1;
         c.needs_fold = 0;
     }
-    leave<G>(d, s, t.rank);
+    if (leave<G>(d, s, t.rank) && fold && t.on) {
+#pragma unroll
+        for (int q = 0; q < PP; ++q) {
+            const unsigned i = pix + (q >> 1) * 2 * G::LR + (q & 1);
+#pragma unroll
+            for (int k = 0; k < 3; ++k) d.eps[k][i] = ep[q][k];
+        }
+    }
 }
 
 // ---------------------------------------------------------------- phase field (Algorithm 1)
 // From the start that FPfInit leaves: v, r, p, a, b, v_con, R and the flags.
 template <int NX, int NY>
-__global__ void __launch_bounds__(RG<NX, NY, 1>::NT, 1) k_res_bccg(const Desc<float>* __restrict__ descs) {
+__global__ void __launch_bounds__(RG<NX, NY, 1>::NT, 1) k_res_bccg(const Desc<float>* __restrict__ descs, long long spin) {
     using G = RG<NX, NY, 1>;
     constexpr int E = G::ER, PP = 2 * E, NT = G::NT, CS = G::CS, W = G::W;
     const Desc<float>& d = descs[blockIdx.y];
@@ -697,7 +734,7 @@ __global__ void __launch_bounds__(RG<NX, NY, 1>::NT, 1) k_res_bccg(const Desc<fl
     __shared__ Shared s;
     __shared__ DF sh[MAXR * W * 32];
     C* sm = reinterpret_cast<C*>(smem_raw);
-    stage<G, NY>(d, s, sm);
+    stage<G, NY>(d, s, sm, spin);
     Lane<G> t;
     lane_setup<NX, NY, 1>(t, d, s, sm);
     const ModeK<float> mk(s.d);
@@ -746,7 +783,8 @@ __global__ void __launch_bounds__(RG<NX, NY, 1>::NT, 1) k_res_bccg(const Desc<fl
         irp = rp != 0.0 ? -1.0 / rp : 0.0;
     };
     C z[E];
-    for (bool first = true; !s.stop && !s.dead; first = false) {
+    bool dead = false;
+    for (bool first = true; !s.stop && !dead; first = false) {
         if (!scalar) {
             if (!first) {   // p = -r + beta p, zero on the active set
                 const float bt = s.beta;
@@ -820,8 +858,8 @@ __global__ void __launch_bounds__(RG<NX, NY, 1>::NT, 1) k_res_bccg(const Desc<fl
             confirm = rec_conv || force;
             force = false;
         }
-        __syncthreads();
-        if (!s.full || s.dead) {
+        dead = sync_dead(s);
+        if (!s.full || dead) {
             if (scalar) {   // beside the next direction's way to the columns
                 nact = __shfl_sync(FULLW, x8, 12);
                 next_dir(x8, 4);
@@ -868,7 +906,7 @@ __global__ void __launch_bounds__(RG<NX, NY, 1>::NT, 1) k_res_bccg(const Desc<fl
                 s.stop = stop;
             }
         }
-        __syncthreads();
+        dead = sync_dead(s);
         if (scalar) {
             last = rr;
             nact = __shfl_sync(FULLW, x8, 8);
@@ -889,7 +927,7 @@ __global__ void __launch_bounds__(RG<NX, NY, 1>::NT, 1) k_res_bccg(const Desc<fl
         c.status |= status;
         c.pf_a = c.pf_b = 1;
     }
-    if (t.on) {
+    if (leave<G>(d, s, t.rank) && t.on) {
 #pragma unroll
         for (int q = 0; q < PP; ++q) {
             const unsigned i = pix + (q >> 1) * 2 * G::LR + (q & 1);
@@ -897,28 +935,24 @@ __global__ void __launch_bounds__(RG<NX, NY, 1>::NT, 1) k_res_bccg(const Desc<fl
             d.flags[i] = fl[q];
         }
     }
-    leave<G>(d, s, t.rank);
 }
 
 // ---------------------------------------------------------------- one Laplacian
 // out = nabla^2 in of one field, in = d.r[0], out = d.q[0] (the allocation-free entry point): the
-// operator alone, without the scalar warp.  A wait that runs out leaves NaN, never a wrong field.
+// operator alone, without the scalar warp.  A wait that runs out in any CTA leaves NaN in all of them, never
+// a wrong field.
 // Bound by its two exchanges and the launch: everything that does not depend on the input (twiddles,
 // lane constants, the cluster's start) runs before the wait for the stream's previous work.  Per call in
 // a row of calls, three passes -> one launch (without the overlap): 16^2 6.1 -> 2.7 us (4.1), 64^2 6.1 ->
 // 2.7 us (6.2), 128^2 7.0 -> 3.7 us (6.2), 256 x 64 7.3 -> 4.0 us (6.2).
 template <int NX, int NY>
-__global__ void __launch_bounds__(RG<NX, NY, 1>::W * 32, 1) k_res_lap(const __grid_constant__ Desc<float> d) {
+__global__ void __launch_bounds__(RG<NX, NY, 1>::W * 32, 1) k_res_lap(const __grid_constant__ Desc<float> d, long long spin) {
     using G = RG<NX, NY, 1>;
     constexpr int E = G::ER;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ Shared s;
     C* sm = reinterpret_cast<C*>(smem_raw);
-    if (threadIdx.x == 0) {
-        s.dead = 0;
-        for (int b = 0; b < 4; ++b) bar_init(s32(&s.bar[b]));
-        asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-    }
+    if (threadIdx.x == 0) init(s, spin);
     Lane<G> t;
     lane_setup<NX, NY, 1>(t, d, s, sm);
     const unsigned pix = (t.rank * G::RPC + t.row) * NX + 2 * t.li;
@@ -933,18 +967,12 @@ __global__ void __launch_bounds__(RG<NX, NY, 1>::W * 32, 1) k_res_lap(const __gr
         z[e] = t.on ? *reinterpret_cast<const C*>(d.r[0] + pix + e * 2 * G::LR) : C{0.f, 0.f};
     unsigned par = 0;
     operate<NX, NY, 1, FColLapPlain>(t, s, sm, mk, z, par, nullptr, [] {});
-    __syncthreads();
-    const bool dead = s.dead;
+    const bool ok = finished<G::CS>(s);
     if (t.on) {
 #pragma unroll
         for (int e = 0; e < E; ++e)
-            *reinterpret_cast<C*>(d.q[0] + pix + e * 2 * G::LR) = dead ? C{NAN, NAN} : z[e];
+            *reinterpret_cast<C*>(d.q[0] + pix + e * 2 * G::LR) = ok ? z[e] : C{NAN, NAN};
     }
-    if (dead) {
-        const long long t0 = clock64();
-        while (clock64() - t0 < 1000000) {}
-    }
-    cluster_sync_all();
 }
 
 // ---------------------------------------------------------------- launch
@@ -954,7 +982,7 @@ __global__ void __launch_bounds__(RG<NX, NY, 1>::W * 32, 1) k_res_lap(const __gr
 constexpr int MAX_DEVICES = 64;
 enum : signed char { UNKNOWN = 0, RUNS = 1, REFUSED = 2 };
 template <typename A>
-cudaError_t go(void (*fn)(A), std::atomic<signed char>* known, int cs, int nt, size_t smem, const A& d, int np,
+cudaError_t go(void (*fn)(A, long long), std::atomic<signed char>* known, int cs, int nt, size_t smem, const A& d, int np,
                cudaStream_t st, bool pdl = false) {
     int dev = 0;
     if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= MAX_DEVICES) return cudaErrorNotSupported;
@@ -984,7 +1012,7 @@ cudaError_t go(void (*fn)(A), std::atomic<signed char>* known, int cs, int nt, s
     }
     if (known[dev] == REFUSED) return cudaErrorNotSupported;
     cfg.numAttrs = pdl ? 2 : 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, fn, d);
+    cudaError_t e = cudaLaunchKernelEx(&cfg, fn, d, barrier_spin_limit());
     if (e == cudaSuccess) count_launch();
     return e;
 }

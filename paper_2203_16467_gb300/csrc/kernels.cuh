@@ -148,6 +148,7 @@ __global__ void __launch_bounds__(EL_NT) k_df(const Desc<T>* __restrict__ descs)
     const Desc<T>& d = descs[blockIdx.y];
     const Consts& k = d.k;
     Ctrl* ctrl = d.ctrl;
+    if (given_up(d)) return;
     constexpr int U = 8;               // pixels of a thread per round
     __shared__ ArgMax sh[EL_NT / 32];
     __shared__ int lov[EL_NT / 32], loD[EL_NT / 32];

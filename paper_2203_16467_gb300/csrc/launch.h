@@ -34,6 +34,8 @@ cudaError_t launch_resident_bccg(const Desc<float>* d, int nx, int ny, int np, c
 // both fields on 8-byte boundaries (a lane moves two adjacent pixels)
 cudaError_t launch_resident_laplacian(const Desc<float>& d, cudaStream_t st);
 inline bool resident_aligned(const void* a, const void* b) { return (((size_t)a | (size_t)b) & 7) == 0; }
+// wait limit of the persistent and the resident kernels in clock cycles
+long long barrier_spin_limit();
 void launch_convert_d2f(float* dst, const double* src, size_t n, cudaStream_t st);
 void launch_convert_f2d(double* dst, const float* src, size_t n, cudaStream_t st);
 

@@ -61,6 +61,10 @@ __device__ __forceinline__ void wdot(Acc<T>& a, T x0, T x1, T x2, T y0, T y1, T 
 
 struct NoCtx {};
 
+// A sub-problem solve of this step was given up (a wait ran out): the rest of the step leaves the state.
+template <typename T>
+__device__ __forceinline__ bool given_up(const Desc<T>& d) { return (ldflag(&d.ctrl->status) & 8) != 0; }
+
 // ---------------------------------------------------------------- mechanics
 template <typename T>
 struct FNewtonIn {   // eps* += theta (rounds > 0), sigma(eps_bar + eps*, phi); FP64: the tangent's frame to q
@@ -423,7 +427,7 @@ struct FPfInit {
         double g; int resc; double eb[3]; double eta_dt; int frozen;
         DF ebf[3], lc, mc, ac, cf, kap;   // double-float: eps_bar, lambda/E, mu/E, eta/dt + c f'', c (AT1) or 2 c (AT2), kappa
     };
-    __device__ static bool skip(const Desc<T>&) { return false; }
+    __device__ static bool skip(const Desc<T>& d) { return given_up(d); }
     __device__ static Ctx prep(const Desc<T>& d) {
         Ctx c;
         c.g = ldd(&d.ctrl->gamma);
@@ -1044,7 +1048,7 @@ template <typename T>
 struct FPost {
     static constexpr int NR = 5;
     struct Ctx { T eb[3]; LameC<T> lm; };
-    __device__ static bool skip(const Desc<T>&) { return false; }
+    __device__ static bool skip(const Desc<T>& d) { return given_up(d); }
     __device__ static Ctx prep(const Desc<T>& d) {
         Ctx c{{}, LameC<T>(d)};
         for (int k = 0; k < 3; ++k) c.eb[k] = T(ldd(&d.ctrl->eps_bar[k]));
