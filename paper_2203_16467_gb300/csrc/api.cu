@@ -1869,17 +1869,24 @@ int pff_batch_step(pff_batch* b, int n_steps, pff_step_report* reports, int* ste
             if (g.np == 1) g.one = h0->ctrl;
             rcs[gi] = run_group_step(g, p, energies, h0);
         };
+        // The groups' own streams start after the caller's stream (what is queued there may read or write the
+        // problems' fields).  A group keeps its stream when it is the last one, so one group waits as well.
+        if (ng > 1 || b->groups[0].stream) {
+            cudaEvent_t ev = nullptr;
+            cudaError_t e = cudaEventCreateWithFlags(&ev, cudaEventDisableTiming);
+            if (e == cudaSuccess) e = cudaEventRecord(ev, b->st);
+            for (auto& bg : b->groups)
+                if (bg.stream && e == cudaSuccess) e = cudaStreamWaitEvent(bg.stream, ev, 0);
+            if (ev) cudaEventDestroy(ev);
+            if (e != cudaSuccess) {   // no such wait: the host's
+                cudaGetLastError();
+                e = cudaStreamSynchronize(b->st);
+                if (e != cudaSuccess) { b->err = cudaGetErrorString(e); return PFF_ERR_CUDA; }
+            }
+        }
         if (ng == 1) {
             run_one(0);
         } else {
-            // the groups' streams start after the caller's stream (copies queued there)
-            cudaEvent_t ev = nullptr;
-            if (cudaEventCreateWithFlags(&ev, cudaEventDisableTiming) == cudaSuccess) {
-                cudaEventRecord(ev, b->st);
-                for (auto& bg : b->groups)
-                    if (bg.stream) cudaStreamWaitEvent(bg.stream, ev, 0);
-                cudaEventDestroy(ev);
-            }
             std::vector<std::thread> th;
             for (int gi = 0; gi < ng; ++gi) th.emplace_back(run_one, gi);
             for (auto& t : th) t.join();
