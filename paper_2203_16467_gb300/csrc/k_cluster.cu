@@ -407,7 +407,7 @@ __global__ void __launch_bounds__(QNT, 1) k_mech_cluster(const Desc<float>* __re
             const double rn = sqrt(R2);
             int stop = 0;
             if (rn <= target || newton_it >= K.max_newton) {
-                if (rn > target) status |= 1;
+                if (!(rn <= target)) status |= 1;   // NaN: not converged
                 stop = 1;
             } else {
                 cg_target = linear ? target : fmax(target, K.mech_cg_rtol * rn);

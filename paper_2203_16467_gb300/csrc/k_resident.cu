@@ -459,9 +459,10 @@ __device__ __forceinline__ double one_sum(Shared& s, const DF* sh, int slot, uns
     send_sum<CS>(s, slot, 0, warp_sum(lane_share<W>(sh, lane)), rank, lane);
     return take_one<CS>(s, slot, parity, lane);
 }
-// x <= y of non-negative doubles (false for a NaN), without the FP64 pipe
+// x <= y of non-negative doubles (false for a NaN in either), without the FP64 pipe
 __device__ __forceinline__ bool le_bits(double x, double y) {
-    return (unsigned long long)__double_as_longlong(x) <= (unsigned long long)__double_as_longlong(y);
+    const unsigned long long a = (unsigned long long)__double_as_longlong(x), b = (unsigned long long)__double_as_longlong(y);
+    return a <= b && b <= 0x7ff0000000000000ull;
 }
 // NR values, value k of every row thread in sh[k 32 W ...] (before a barrier): each warp sums some of them.
 template <int NR, int W, int CS>

@@ -136,7 +136,7 @@ struct FNewtonOut {   // R = P sigma; CG start r = p = -R, theta = 0; Newton tes
         c->mech_target = target;
         c->R2 = R2;
         if (rn <= target || c->newton_it >= k.max_newton) {
-            if (rn > target) c->status |= 1;
+            if (!(rn <= target)) c->status |= 1;   // NaN: not converged
             c->nd_a = 1;
             c->cg_a = 1;
             c->cg_b = 1;
