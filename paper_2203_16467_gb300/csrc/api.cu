@@ -526,7 +526,7 @@ static int g_persist_share = 8;    // the persistent launch takes 1/share of the
 static bool bccg_chain(const Group& g) { return g.precond || g_bccg4.load(); }
 // chunks that hold every iteration a solve may take
 static int bccg_chunks(const Group& g, int max_pf) {
-    return bccg_chain(g) ? max_pf / CHUNK + 2 : (2 * max_pf) / SLOTS + 2;
+    return bccg_chain(g) ? max_pf / CHUNK + 2 : max_pf / (SLOTS / 2) + 2;
 }
 
 template <typename T>
