@@ -34,6 +34,25 @@ __host__ __device__ __forceinline__ int driving_of(int split) {
 enum { CRACK_SET = 0, DAMAGE = 1 };
 
 // ---------------------------------------------------------------------------
+// A quotient a / x whose divisor is known earlier than its dividend: 1 / (x s) = hi + lo is formed off the
+// chain (an FP64 division takes 550 cycles, a product 65), and (a s) hi + (a s) lo rounds once, so the
+// quotient is as accurate as a division (its error is half a unit and some 2^-50 of one; 2e5 random
+// quotients all equal the division's).  s, a power of two, keeps the parts within the exponent range.  The
+// quotient by 0 is 0.
+struct Recip { double hi, lo, s; };
+__device__ __forceinline__ Recip recip(double x) {
+    const unsigned e = ((unsigned)__double2hiint(x) >> 20) & 0x7ffu;   // biased exponent
+    const double s = e < 64u ? 0x1p256 : e > 1982u ? 0x1p-256 : 1.0;
+    const double xs = x * s, hi = 1.0 / xs, lo = fma(-hi, xs, 1.0) * hi;
+    const bool in = e < 0x7ffu && x != 0.0;
+    return Recip{x != 0.0 ? hi : 0.0, in ? lo : 0.0, s};
+}
+__device__ __forceinline__ double quotient(double a, const Recip& r) {
+    a *= r.s;
+    return fma(a, r.hi, a * r.lo);
+}
+
+// ---------------------------------------------------------------------------
 // Control block of one problem (device memory).  Scalars of the iterative
 // solvers live here so that kernels chain without host round trips.  Flags
 // come in pairs (x_a, x_b): a kernel never writes a flag that kernels of the
@@ -44,16 +63,16 @@ struct Ctrl {
     double sumE2;           // sum of E^2 over pixels (scale of the mechanics tolerance)
     double sumE;            // sum of E
     // mechanics
-    double mech_target, R2, rr, pAp, rAp, qq, alpha, beta, cg_target;
-    double rr_inv;          // 1 / rr (0 for rr = 0), formed beside alpha
+    double mech_target, R2, rr, alpha, beta, cg_target;
+    Recip rr_inv;           // of rr, formed beside alpha
     int nd_a, nd_b, newton_it, needs_fold;
     int cg_a, cg_b, cg_it, cg_total, cg_break;
     // near-equilibrium rescale (Algorithm 4 lines 4-10)
     double mF_max, D_max, Rf_star, D_star, gamma;
     int istar, flag, rescaled;
     // phase field (Algorithm 1)
-    double pf_rr, pf_rp, pJp, pf_alpha, pf_beta, pf_target, pf_best;   // pf_best, pf_last_full: squared norms
-    double pf_irp;          // -1 / (r.p) of the direction, formed beside alpha
+    double pf_rr, pf_rp, pf_alpha, pf_beta, pf_target, pf_best;   // pf_best, pf_last_full: squared norms
+    Recip pf_irp;           // of -r.p of the direction, formed beside alpha
     double pf_pap;          // sum a p^2 of the direction (the diagonal part of p.Jp)
     int pf_a, pf_b, pf_it, pf_break, n_active, pf_best_it, pf_clamp_iters;
     // residual recurrence: pf_full = this iteration evaluates Jv explicitly
@@ -77,6 +96,9 @@ struct Ctrl {
     int post_mode;          // 0: post-step applies Algorithm 4's strain increment; 1: host decides
     int pad;
 };
+// The last block of a reduction moves the control block with 128 threads in one go, a word each (a second
+// round trip costs 3 % of a 512^2 BCCG solve).
+static_assert(sizeof(Ctrl) <= 512, "one word per thread of the smallest block");
 
 // Model constants of a problem, resolved on the host.
 struct Consts {

@@ -570,7 +570,8 @@ __global__ void __launch_bounds__(RG<NX, NY, 3>::NT, 1) k_res_mech(const Desc<fl
     unsigned par = 0, p0 = 0, p1 = 0;   // parities: modes and rows, sums slot 0, sums slot 1
     // The scalar warp's state (the same in its lanes): FNewtonOut, FCgIn and FCgOut with norms compared
     // by their squares, the divisions off the chain of the iteration, and no control block between.
-    double target = 0.0, target2 = 0.0, cg2 = 0.0, R2 = 0.0, rr = 0.0, rr_inv = 0.0;
+    double target = 0.0, target2 = 0.0, cg2 = 0.0, R2 = 0.0, rr = 0.0;
+    Recip rr_inv{0.0, 0.0, 1.0};
     int cg_it = 0, cg_total = 0, newton_it = 0, status = 0;
     if (scalar) {
         const Consts& k = s.d.k;
@@ -659,7 +660,7 @@ __global__ void __launch_bounds__(RG<NX, NY, 3>::NT, 1) k_res_mech(const Desc<fl
                 const double pAp = one_sum<W, CS>(s, sh, 0, p0, t.rank, t.lane);
                 p0 ^= 1u;
                 const bool go_on = pAp > 0.0;
-                rr_inv = rr > 0.0 ? 1.0 / rr : 0.0;
+                rr_inv = recip(rr);
                 const float alpha = go_on ? (float)(rr / pAp) : 0.f;
                 if (t.lane == 0) {
                     s.alpha = alpha;
@@ -687,7 +688,7 @@ __global__ void __launch_bounds__(RG<NX, NY, 3>::NT, 1) k_res_mech(const Desc<fl
             if (scalar) {
                 rr = one_sum<W, CS>(s, sh, 1, p1, t.rank, t.lane);
                 p1 ^= 1u;
-                const float beta = (float)(rr * rr_inv);
+                const float beta = (float)quotient(rr, rr_inv);
                 ++cg_it;
                 ++cg_total;
                 const bool conv = le_bits(rr, cg2), stop = conv || cg_it >= s.d.k.max_cg;
@@ -760,7 +761,8 @@ __global__ void __launch_bounds__(RG<NX, NY, 1>::NT, 1) k_res_bccg(const Desc<fl
     unsigned par = 0, p0 = 0, p1 = 0;
     // The scalar warp's state (the same in its lanes): FColLapPFQ's and FPfSlotOut's finalizers with
     // the next step's flags and beta first and everything else after the row warps have gone on.
-    double target2 = 0.0, kin = 0.0, pap = 0.0, rp = 0.0, irp = 0.0, beta = 0.0, rr = 0.0, best = 0.0, last = 0.0, nact = 0.0;
+    double target2 = 0.0, kin = 0.0, pap = 0.0, rp = 0.0, beta = 0.0, rr = 0.0, best = 0.0, last = 0.0, nact = 0.0;
+    Recip irp{0.0, 0.0, 1.0};   // of -rp
     int it = 0, best_it = 0, since_full = 0, full_iters = 0, clamp_iters = 0, status = 0;
     bool force = false, confirm = false, broke = false;
     if (scalar) {
@@ -769,7 +771,7 @@ __global__ void __launch_bounds__(RG<NX, NY, 1>::NT, 1) k_res_bccg(const Desc<fl
         kin = s.d.k.kappa * s.d.k.inv_n;
         pap = c.pf_pap;
         rp = c.pf_rp;
-        irp = rp != 0.0 ? -1.0 / rp : 0.0;
+        irp = recip(-rp);
         rr = c.pf_rr;
         best = last = rr;
         if (t.lane == 0) s.stop = c.pf_b;
@@ -781,7 +783,7 @@ __global__ void __launch_bounds__(RG<NX, NY, 1>::NT, 1) k_res_bccg(const Desc<fl
                      S2 = __shfl_sync(FULLW, x, 4 * k0 + 8), S3 = __shfl_sync(FULLW, x, 4 * k0 + 12);
         pap = S0 - 2.0 * beta * S1 + beta * beta * S2;
         rp = -rr + beta * S3;
-        irp = rp != 0.0 ? -1.0 / rp : 0.0;
+        irp = recip(-rp);
     };
     C z[E];
     bool dead = false;
@@ -841,7 +843,7 @@ __global__ void __launch_bounds__(RG<NX, NY, 1>::NT, 1) k_res_bccg(const Desc<fl
             full_now = clamped || rec_conv || force || since_full + 1 >= PF_REFRESH;
             bool stop = false;
             if (!full_now) {
-                beta = (r2 - rro) * irp;
+                beta = quotient(r2 - rro, irp);
                 rr = r2;
                 ++it;
                 ++since_full;
@@ -890,7 +892,7 @@ __global__ void __launch_bounds__(RG<NX, NY, 1>::NT, 1) k_res_bccg(const Desc<fl
             x8 = take_many<7, CS>(s, 1, p1, t.lane);
             p1 ^= 1u;
             rr = __shfl_sync(FULLW, x8, 0);
-            beta = (rr - __shfl_sync(FULLW, x8, 4)) * irp;
+            beta = quotient(rr - __shfl_sync(FULLW, x8, 4), irp);
             ++it;
             ++full_iters;
             since_full = 0;

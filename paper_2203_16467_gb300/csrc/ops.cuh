@@ -227,7 +227,6 @@ struct FCgIn {
     __device__ static void finalize(const Desc<T>& d, const double* tot) {
         Ctrl* c = d.ctrl;
         const double pAp = tot[0];
-        c->pAp = pAp;
         if (!(pAp > 0.0)) {   // p.Ap <= 0: stop (A8); every block has read cg_b already
             c->cg_break = 1;
             c->alpha = 0.0;
@@ -235,9 +234,7 @@ struct FCgIn {
             c->cg_b = 1;
         } else {
             c->alpha = c->rr / pAp;
-            // for FCgOut's beta, whose finalizer ends the iteration's chain (an FP64 division takes
-            // 550 cycles, a square root 600, a product 65)
-            c->rr_inv = c->rr > 0.0 ? 1.0 / c->rr : 0.0;
+            c->rr_inv = recip(c->rr);   // for FCgOut's beta, whose finalizer ends the iteration's chain
         }
     }
 };
@@ -277,7 +274,7 @@ struct FCgOut {
         const double rr = tot[0];
         c->cg_it += 1;
         c->cg_total += 1;
-        c->beta = rr * c->rr_inv;
+        c->beta = quotient(rr, c->rr_inv);
         c->rr = rr;
         const bool conv = rr <= c->cg_target * c->cg_target;
         if (conv || c->cg_it >= d.k.max_cg) {
@@ -663,9 +660,8 @@ struct FPfA3 {   // J p; p.Jp, r.p -> alpha = -(r.p)/(p.Jp)
     }
     __device__ static void finalize(const Desc<T>& d, const double* tot) {
         Ctrl* c = d.ctrl;
-        c->pJp = tot[0];
         c->pf_rp = tot[1];
-        c->pf_irp = tot[1] != 0.0 ? -1.0 / tot[1] : 0.0;
+        c->pf_irp = recip(-tot[1]);
         if (!(tot[0] > 0.0)) {
             c->pf_break = 1;
             c->pf_alpha = 0.0;
@@ -711,15 +707,15 @@ struct FColLapPFQ {   // (as such the column pass of the cluster-resident solve)
     }
     template <typename T> __device__ static void finalize(const Desc<T>& d, const double* tot) {
         Ctrl* c = d.ctrl;
+        const Recip irp = recip(-c->pf_rp);   // for the beta of this iteration
         const double pJp = c->pf_pap + d.k.kappa * tot[0] * d.k.inv_n;
-        c->pJp = pJp;
+        c->pf_irp = irp;
         if (!(pJp > 0.0)) {
             c->pf_break = 1;
             c->pf_alpha = 0.0;
         } else {
             c->pf_alpha = -c->pf_rp / pJp;
         }
-        c->pf_irp = c->pf_rp != 0.0 ? -1.0 / c->pf_rp : 0.0;   // for the beta of this iteration
     }
 };
 
@@ -735,7 +731,7 @@ __device__ __forceinline__ void pf_next_dir(Ctrl* c, const double* S) {
 template <typename T>
 __device__ __forceinline__ void pf_finish(const Desc<T>& d, Ctrl* c, double rr, double rro, double nact, bool full) {
     // (the preconditioned variant takes beta from the z pass); -r.p = alpha p.Jp
-    if (!d.k.pf_precond) c->pf_beta = (rr - rro) * c->pf_irp;
+    if (!d.k.pf_precond) c->pf_beta = quotient(rr - rro, c->pf_irp);
     c->pf_rr = rr;
     c->pf_it += 1;
     c->n_active = (int)nact;
