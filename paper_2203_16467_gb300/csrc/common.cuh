@@ -508,15 +508,20 @@ __device__ __forceinline__ T psi_voldev(T xx, T yy, T xy, T lam, T mu) {
 }
 
 // psi_0^+ of the crack-driving-force model in double-float arithmetic, for FP32 problems (GB300 runs
-// FP64 at 1/64 of the FP32 rate).  `small`: the operands are too near the ends of the FP32 exponent
-// range for the low parts (the caller then takes the FP64 function).
+// FP64 at 1/64 of the FP32 rate).  With M the largest |eps_bar| + |eps*| of the components, the value is off
+// by less than 2^-41 (2 |lambda| + 10 mu) M^2 (df_psi_size): an addition's error is at most 5 2^-48 of its
+// operands' magnitudes, a product's 7 2^-48, the root's 51 2^-48 of itself, and the longest path (spectral)
+// adds up to 83 2^-48 of that size.  df_psi_range: no part leaves the FP32 exponent range (else the caller
+// takes the FP64 function).
 struct DF3 { DF xx, yy, xy; };
 __device__ __forceinline__ DF df_pos(DF a) { return a.hi > 0.f ? a : DF{0.f, 0.f}; }
-__device__ __forceinline__ bool df_psi_range(const DF3& e, float lam, float mu) {
-    const float m = fmaxf(fmaxf(fabsf(e.xx.hi), fabsf(e.yy.hi)), fabsf(e.xy.hi));
+__device__ __forceinline__ bool df_psi_range(float M, float lam, float mu) {
     const float k = fmaxf(fabsf(lam), mu);
-    return m > 1e-10f && m < 1e10f && k > 1e-15f && k < 1e15f;
+    return M > 1e-8f && M < 1e10f && k > 1e-15f && k < 1e15f;
 }
+__device__ __forceinline__ float df_psi_size(float M, float lam, float mu) { return (2.f * fabsf(lam) + 10.f * mu) * M * M; }
+// are all values within err of hi + lo rounded to the same FP32 number (false for a NaN)
+__device__ __forceinline__ bool df_rounds(DF x, float err) { return x.hi + (x.lo - err) == x.hi + (x.lo + err); }
 __device__ __forceinline__ DF df_psi_plus(int split, const DF3& e, DF lam, DF mu) {
     const int s = driving_of(split);
     const DF tr = df_add(e.xx, e.yy);

@@ -411,9 +411,12 @@ struct FCopyOut {
 // v_con = phi_con(phi_n) - phi_n <= 0; v^0 = 0; r^0 = -b masked; p^0 = -r^0.
 //
 // psi_0^+, a and b are formed in FP64 and stored in the problem's precision.  FP32 problems form them
-// in double-float arithmetic instead (the same FP32 values but for one in some 2^20; FP64 only near
-// the ends of the FP32 exponent range): the FP64 pipe bound this kernel (one 512^2 problem 39 -> 19 us,
-// eight 213 -> 77 us, 2048^2 410 -> 142 us; now the issue of some 400 instructions per pixel).
+// in double-float arithmetic with a bound of its error: where every value within the bound rounds to one
+// FP32 number, that is what FP64 gives as well; elsewhere (a pixel in some thousands, more where b is a small
+// difference; and near the ends of the FP32 exponent range) the pixel is evaluated in FP64.  So the stored
+// values are those of FP64 arithmetic, whose pipe bound this kernel: one 512^2 problem 39 -> 23 us, eight
+// 213 -> 93 us, 2048^2 410 -> 156 us (175 with AT2), now the issue of some 400 instructions per pixel (the
+// double-float values alone, off by one in some 2^20 and more where b cancels: 18, 73 and 142 us).
 static __device__ __noinline__ double psi_plus_fp64(int split, double xx, double yy, double xy, double lam, double mu) {
     return psi_plus<double>(split, xx, yy, xy, lam, mu);
 }
@@ -442,6 +445,16 @@ struct FPfInit {
         }
         return c;
     }
+    __device__ __forceinline__ static void fp64(const Consts& k, const Ctx& c, T e0, T e1, T e2, T E, T ph, T lap, T& a, T& b) {
+        const double Ed = (double)E, phd = (double)ph, lam = k.lam_c * Ed, mu = k.mu_c * Ed;
+        const double xx = c.eb[0] + (double)e0, yy = c.eb[1] + (double)e1, xy = c.eb[2] + (double)e2;
+        double psi;
+        if constexpr (sizeof(T) == 4) psi = psi_plus_fp64(k.split, xx, yy, xy, lam, mu);
+        else psi = psi_plus<double>(k.split, xx, yy, xy, lam, mu);
+        const double fp = k.fracture == AT1 ? 1.0 : 2.0 * phd;
+        a = T(c.eta_dt + 2.0 * psi + k.cf2);
+        b = T(2.0 * (1.0 - phd) * psi - k.c * fp + k.kappa * (double)lap);
+    }
     __device__ static void pixel(const Desc<T>& d, const Ctx& c, size_t i, Acc<T>* acc) {
         const Consts& k = d.k;
         T e0 = d.eps[0][i], e1 = d.eps[1][i], e2 = d.eps[2][i];
@@ -450,33 +463,27 @@ struct FPfInit {
             e0 *= g; e1 *= g; e2 *= g;
             d.eps[0][i] = e0; d.eps[1][i] = e1; d.eps[2][i] = e2;
         }
-        T ph = d.phi[i];
+        const T E = d.E[i], ph = d.phi[i], lap = d.lap[i];
         T a, b;
+        bool done = false;
         if constexpr (sizeof(T) == 4) {
-            const float E = d.E[i], lap = d.lap[i];
             const DF3 e{df_add(c.ebf[0], DF{e0, 0.f}), df_add(c.ebf[1], DF{e1, 0.f}), df_add(c.ebf[2], DF{e2, 0.f})};
             const DF lam = df_mulf(c.lc, E), mu = df_mulf(c.mc, E);
-            DF psi2;
-            if (df_psi_range(e, lam.hi, mu.hi))
-                psi2 = df_scale(df_psi_plus(k.split, e, lam, mu), 2.f);
-            else
-                psi2 = df_of(2.0 * psi_plus_fp64(k.split, c.eb[0] + (double)e0, c.eb[1] + (double)e1, c.eb[2] + (double)e2,
-                                                 k.lam_c * (double)E, k.mu_c * (double)E));
+            const float M = fmaxf(fmaxf(fabsf(c.ebf[0].hi) + fabsf(e0), fabsf(c.ebf[1].hi) + fabsf(e1)),
+                                  fabsf(c.ebf[2].hi) + fabsf(e2));
+            const DF psi2 = df_scale(df_psi_plus(k.split, e, lam, mu), 2.f);
+            const DF g = df_sum(1.f, -ph), cf = k.fracture == AT1 ? c.cf : df_mulf(c.cf, ph), kl = df_mulf(c.kap, lap);
             const DF av = df_add(c.ac, psi2);
-            DF bv = df_mul(df_sum(1.f, -ph), psi2);
-            bv = df_add(bv, df_neg(k.fracture == AT1 ? c.cf : df_mulf(c.cf, ph)));
-            bv = df_add(bv, df_mulf(c.kap, lap));
+            const DF bv = df_add(df_add(df_mul(g, psi2), df_neg(cf)), kl);
+            // bounds of the errors: 2^-41 of the size of the terms (FP64's own error is far within)
+            const float u = 4.5474735e-13f, s2 = 2.f * df_psi_size(M, lam.hi, mu.hi);
+            const float ea = fmaf(u, s2 + fabsf(c.ac.hi), 1e-38f);
+            const float eb = fmaf(u, fabsf(g.hi) * s2 + fabsf(cf.hi) + fabsf(kl.hi), 1e-38f);
             a = av.hi + av.lo;
             b = bv.hi + bv.lo;
-        } else {
-            double E = (double)d.E[i];
-            double lam = k.lam_c * E, mu = k.mu_c * E;
-            double psi = psi_plus<double>(k.split, c.eb[0] + (double)e0, c.eb[1] + (double)e1, c.eb[2] + (double)e2, lam, mu);
-            double phd = (double)ph;
-            double fp = k.fracture == AT1 ? 1.0 : 2.0 * phd;
-            a = T(c.eta_dt + 2.0 * psi + k.cf2);
-            b = T(2.0 * (1.0 - phd) * psi - k.c * fp + k.kappa * (double)d.lap[i]);
+            done = df_psi_range(M, lam.hi, mu.hi) && df_rounds(av, ea) && df_rounds(bv, eb);
         }
+        if (!done) fp64(k, c, e0, e1, e2, E, ph, lap, a, b);
         T pcon = c.frozen ? d.aux[i] : ((k.irrev == CRACK_SET) ? (ph >= T(k.crack_thr) ? ph : T(0)) : ph);
         T vcon = pcon - ph;
         T v = T(0) < vcon ? vcon : T(0);
