@@ -764,7 +764,7 @@ __global__ void __launch_bounds__(RG<NX, NY, 1>::NT, 1) k_res_bccg(const Desc<fl
     double target2 = 0.0, kin = 0.0, pap = 0.0, rp = 0.0, beta = 0.0, rr = 0.0, best = 0.0, last = 0.0, nact = 0.0;
     Recip irp{0.0, 0.0, 1.0};   // of -rp
     int it = 0, best_it = 0, since_full = 0, full_iters = 0, clamp_iters = 0, status = 0;
-    bool force = false, confirm = false, broke = false;
+    bool confirm = false, broke = false;
     if (scalar) {
         const Ctrl& c = s.ctrl;
         target2 = c.pf_target * c.pf_target;
@@ -840,7 +840,7 @@ __global__ void __launch_bounds__(RG<NX, NY, 1>::NT, 1) k_res_bccg(const Desc<fl
             const double r2 = __shfl_sync(FULLW, x8, 4), rro = __shfl_sync(FULLW, x8, 8);
             const bool clamped = __double_as_longlong(__shfl_sync(FULLW, x8, 0)) > 0;
             const bool rec_conv = le_bits(r2, target2);
-            full_now = clamped || rec_conv || force || since_full + 1 >= PF_REFRESH;
+            full_now = clamped || rec_conv || since_full + 1 >= PF_REFRESH;
             bool stop = false;
             if (!full_now) {
                 beta = quotient(r2 - rro, irp);
@@ -858,8 +858,7 @@ __global__ void __launch_bounds__(RG<NX, NY, 1>::NT, 1) k_res_bccg(const Desc<fl
                 s.stop = stop;
             }
             clamp_iters += clamped;
-            confirm = rec_conv || force;
-            force = false;
+            confirm = rec_conv;
         }
         dead = sync_dead(s);
         if (!s.full || dead) {
