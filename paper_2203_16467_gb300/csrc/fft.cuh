@@ -876,19 +876,24 @@ struct Col16Cfg {
     static constexpr size_t SMEM = (size_t)NC * CW * XS * sizeof(typename CT<T>::t);
 };
 
-// u[c][at(r)] *= w^r for r = 1 .. 15 (w^1, w^2, w^4, w^8 from the table tw[r step], the others products)
-template <typename C, int NC, bool CONJ, bool PERM>
+// u[c][at(r)] *= w^r for r = 1 .. 15.  TABLE: all from the table tw[r step]; else w^1, w^2, w^3, w^4, w^8,
+// w^12, and the others as products of two of these.  Products of three (from w^1, w^2, w^4, w^8) made the
+// Laplacian of a field with 1024 rows 8 % and with 2048 rows 4 % less accurate than the Stockham pass; now they
+// are 4 % and 2 % more accurate.  With 2048 points the whole table costs 5 % of a load step (registers), with
+// 1024 points 0.9 % (1024^2 4330 -> 4367 us), the products there 0.5 % of accuracy.
+template <typename C, int NC, bool CONJ, bool PERM, bool TABLE>
 __device__ __forceinline__ void twiddle16(C (&u)[NC][16], const C* tw, int step) {
+    auto from_table = [](int r) { return TABLE || r < 4 || r % 4 == 0; };
     C w[16];
 #pragma unroll
-    for (int r = 1; r < 16; r *= 2) {
+    for (int r = 1; r < 16; ++r) {
+        if (!from_table(r)) continue;
         const C x = __ldg(tw + r * step);
         w[r] = CONJ ? C{x.x, -x.y} : x;
     }
 #pragma unroll
     for (int r = 1; r < 16; ++r) {
-        const int hi = r >= 8 ? 8 : r >= 4 ? 4 : r >= 2 ? 2 : 1;
-        if (r != hi) w[r] = cmul(w[hi], w[r - hi]);
+        if (!from_table(r)) w[r] = cmul(w[r & ~3], w[r & 3]);
 #pragma unroll
         for (int c = 0; c < NC; ++c) {
             C& x = u[c][PERM ? at16(r) : r];
@@ -923,7 +928,7 @@ __global__ void __launch_bounds__(CW * NY / 16, NC == 1 && NY == 2048 ? 2 : 1) k
     // forward
 #pragma unroll
     for (int c = 0; c < NC; ++c) dft16<C, false>(u[c]);
-    twiddle16<C, NC, false, true>(u, tw, t);
+    twiddle16<C, NC, false, true, NY == 1024>(u, tw, t);
 #pragma unroll
     for (int c = 0; c < NC; ++c)
 #pragma unroll
@@ -935,7 +940,7 @@ __global__ void __launch_bounds__(CW * NY / 16, NC == 1 && NY == 2048 ? 2 : 1) k
         for (int b = 0; b < 16; ++b) u[c][b] = xb[c * CS + P1 * k1 + a + R3 * b];
         dft16<C, false>(u[c]);
     }
-    twiddle16<C, NC, false, true>(u, tw, 16 * a);
+    twiddle16<C, NC, false, true, NY == 1024>(u, tw, 16 * a);
     __syncthreads();
 #pragma unroll
     for (int c = 0; c < NC; ++c)
@@ -982,7 +987,7 @@ __global__ void __launch_bounds__(CW * NY / 16, NC == 1 && NY == 2048 ? 2 : 1) k
     for (int c = 0; c < NC; ++c)
 #pragma unroll
         for (int k = 0; k < 16; ++k) u[c][k] = xb[c * CS + P2 * a + 16 * k + k1];
-    twiddle16<C, NC, true, false>(u, tw, 16 * a);
+    twiddle16<C, NC, true, false, NY == 1024>(u, tw, 16 * a);
     __syncthreads();
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
@@ -995,7 +1000,7 @@ __global__ void __launch_bounds__(CW * NY / 16, NC == 1 && NY == 2048 ? 2 : 1) k
     for (int c = 0; c < NC; ++c)
 #pragma unroll
         for (int k = 0; k < 16; ++k) u[c][k] = xb[c * CS + P1 * k + t];
-    twiddle16<C, NC, true, false>(u, tw, t);
+    twiddle16<C, NC, true, false, NY == 1024>(u, tw, t);
 #pragma unroll
     for (int c = 0; c < NC; ++c) {
         dft16<C, true>(u[c]);
