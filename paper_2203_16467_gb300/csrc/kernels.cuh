@@ -430,14 +430,16 @@ void go_col(const Desc<T>* d, int np, int nm, cudaStream_t st, int key) {
         default: break;                             \
     }
 
-// Up to 256^2 one pixel per thread, so that a small grid's few pixels spread over the SMs (64^2: the
-// BCCG start 24 -> 13 us, post-step 16 -> 14 us; 256^2: 26 -> 13 us); four per thread, whose loads
-// are in flight together, beyond (one per thread at 512^2: post-step of one simulation 18 -> 23 us, of
-// eight 46 -> 75 us, for the reductions of four times the blocks).  The number of problems does not
-// enter: the summation order, and with it every bit, is the same in every launch group.
+// Up to 2^14 pixels one pixel per thread, so that a small grid's few pixels spread over the SMs (64^2: the
+// BCCG start 24 -> 13 us, post-step 16 -> 14 us; load steps of 64^2 and 128^2 1 % faster, groups of 64 of
+// them 0 to 2 % slower); four per thread, whose loads are in flight together, beyond: one per thread has four
+// times the blocks and block reductions (load step of a single 256^2 3139 -> 3132 us, but of 64 of them in
+// groups of eight 20.39 -> 20.80 ms, in one group 23.47 -> 23.89; eight 512^2: post-step 46 -> 75 us).  The
+// number of problems does not enter: the summation order, and with it every bit, is the same in every launch
+// group.
 inline int elem_blocks(int nx, int ny) {
     const long long n = (long long)nx * ny, one = (n + EL_NT - 1) / EL_NT;
-    const long long b = one <= 256 ? one : (n + EL_NT * 4 - 1) / (EL_NT * 4);
+    const long long b = one <= 64 ? one : (n + EL_NT * 4 - 1) / (EL_NT * 4);
     return (int)(b > 2048 ? 2048 : b < 1 ? 1 : b);
 }
 
