@@ -504,7 +504,8 @@ static bool mech_cluster_group(const Group& g) {
 // A sub-problem solve of a group of small FP32 grids in one launch, a cluster per problem
 // (k_resident.cu; kind 0 mechanics, 1 phase field).  The per-kernel path stays for other sizes,
 // FP64, the preconditioned and the four-pass BCCG and kernel timing (which times its kernels), and
-// where the device cannot host the cluster: false, nothing launched.
+// where the device cannot host the cluster: false, nothing launched.  The size alone decides, not the
+// number of problems (both sides are measured in k_resident.cu).
 template <typename T>
 static bool resident_solve(int kind, const Group& g) {
     if constexpr (sizeof(T) == 4) {

@@ -3,13 +3,20 @@
 // state on chip.
 //
 // Why.  At these sizes the kernels of an iteration hold well under a microsecond of work each and
-// cost 6-10 us (launch, control block read, load latency, reduction tail).  One mechanics solve from
-// eps* = 0 / one BCCG solve / one load step, per-kernel path -> here, us, host calls included:
-// 16^2 981 -> 193 / 1746 -> 378 / 2474 -> 471; 64^2 2163 -> 461 / 2377 -> 511 / 3171 -> 652; 128^2
-// 1696 -> 866 / 2988 -> 727 / 3724 -> 1195; 16 problems of 128^2 in one group 6682 -> 4311 per load step.
-// At 256^2 the 16 SMs of a cluster no longer keep up with the whole chip (64 problems of 256^2 in
-// groups of eight, 40 against 27 ms per load step), hence the limit of 2^14 pixels.  A cluster exchanges
-// through its own shared memory instead:
+// cost 6-10 us (launch, control block read, load latency, reduction tail).  One load step, per-kernel path
+// -> here, us, host calls included: 16^2 1845 -> 528, 64^2 2468 -> 671, 128^2 2953 -> 1092, 64 x 256 3293 ->
+// 1516.  At 256^2 the 16 SMs of a cluster no longer keep up with the whole chip (64 problems of 256^2 in
+// groups of eight, 40 against 20 ms per load step), hence the limit of 2^14 pixels.
+// A cluster has its SMs to itself (at 2^14 pixels a CTA's registers fill one), so the chip runs nine
+// clusters of 16 at a time and a group's others queue, while the per-kernel path hardly slows until a launch
+// holds some 2^19 pixels.  Groups in one launch, per-kernel -> here, ms: 64^2 64 problems 7.0 -> 6.1, 128 11.4
+// -> 11.9; 128^2 16 4.9 -> 3.5, 32 6.6 -> 6.1, 64 10.5 -> 11.9; 64 x 256 16 4.9 -> 4.6, 32 6.6 -> 8.0, 64 10.3 ->
+// 15.0.  Groups of one in streams are faster here throughout (64 of 128^2 26.2 -> 13.2).  The number of
+// problems still does not choose the path: the two differ in the last bits, and a simulation's result must not
+// depend on the grouping of its batch (pff_batch_autotune changes that as it goes).
+// (Registers: the 17 warps at 64 x 256 leave 96 a thread, which spills 716 bytes in the mechanics solve and 248
+// in the BCCG; the nine warps at 128^2 leave 168, which spills 160 bytes in the mechanics solve.)
+// A cluster exchanges through its own shared memory instead:
 //   rows     CTA c owns the rows [c RPC, (c+1) RPC), a row per warp (several short rows); the vectors
 //            of the iteration (p, r, theta, or p, r, v, R) of its pixels and the constants stay in
 //            registers for the whole solve;
@@ -944,9 +951,10 @@ __global__ void __launch_bounds__(RG<NX, NY, 1>::NT, 1) k_res_bccg(const Desc<fl
 // operator alone, without the scalar warp.  A wait that runs out in any CTA leaves NaN in all of them, never
 // a wrong field.
 // Bound by its two exchanges and the launch: everything that does not depend on the input (twiddles,
-// lane constants, the cluster's start) runs before the wait for the stream's previous work.  Per call in
-// a row of calls, three passes -> one launch (without the overlap): 16^2 6.1 -> 2.7 us (4.1), 64^2 6.1 ->
-// 2.7 us (6.2), 128^2 7.0 -> 3.7 us (6.2), 256 x 64 7.3 -> 4.0 us (6.2).
+// lane constants, the cluster's start) runs before the wait for the stream's previous work.  The rate of a
+// row of calls, whose prologues overlap, three passes -> one launch: 16^2 6.1 -> 2.6 us, 64^2 5.9 -> 2.7, 128^2
+// 6.8 -> 3.7, 256 x 64 6.6 -> 4.0.  One call that is waited for (host call, launch and wait included): 16^2 14.2
+// -> 12.1 us, 64^2 15.5 -> 12.9, 128^2 16.8 -> 14.2, 256 x 64 16.7 -> 14.5.
 template <int NX, int NY>
 __global__ void __launch_bounds__(RG<NX, NY, 1>::W * 32, 1) k_res_lap(const __grid_constant__ Desc<float> d, long long spin) {
     using G = RG<NX, NY, 1>;

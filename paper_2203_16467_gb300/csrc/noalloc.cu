@@ -13,9 +13,9 @@
 // A call is launch-bound (a 64^2 field holds under a microsecond of work), so the
 // descriptor is a kernel argument (its copy to the device was a fourth operation
 // in the stream), and FP32 fields up to 2^14 pixels take one launch of one
-// cluster (k_resident.cu): 64^2 FP32 11.3 -> 2.7 us per call (6.1 with the
-// argument alone), 512 x 256 FP64 49 -> 45 us (now 43; the FP64 pipe bounds its
-// passes).
+// cluster (k_resident.cu): a 64^2 FP32 call in a row of calls 11.3 -> 2.7 us (5.9
+// with the argument alone), one that is waited for 12.9 us (15.5), 512 x 256 FP64
+// 49 -> 45 us (now 43; the FP64 pipe bounds its passes).
 #include <cmath>
 #include <cstring>
 #include <mutex>

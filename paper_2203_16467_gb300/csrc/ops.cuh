@@ -6,7 +6,9 @@
 //   K2 col      FColGamma : Gamma projection between column FFTs
 //   K3 row_inv  FCgOut    : q = A p; x += a p, r -= a q; explicit r.r -> stop test, b
 // Newton residual (Eq. elasticity_nodal): FNewtonIn / FColGammaN / FNewtonOut.
-// Phase field (Algorithm 1), two operator applications per BCCG iteration:
+// Phase field (Algorithm 1): FPfInit, then one operator application per BCCG iteration and one more where
+// J v - b is evaluated explicitly, both by the same three kernels (FPfSlotIn / FColLapPFS / FPfSlotOut).
+// The preconditioned and the four-pass variants and the persistent kernel instead:
 //   A1 FPfA1 (p = -r + b p, masked) -> A2 lap -> A3 FPfA3 (p.Jp, r.p -> alpha)
 //   B1 FPfB1 (v = max(v + alpha p, v_con)) -> B2 lap -> B3 FPfB3 (r = Jv - b, active set,
 //   r.r, r.r_old -> beta, convergence).
