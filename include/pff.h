@@ -419,10 +419,11 @@ int pff_set_pdl(int on);
  * problem, or a batch group of one) in one persistent cooperative launch
  * (default off): the BCCG iterations of Algorithm 1 run without kernel
  * boundaries, their phases separated by grid barriers that carry the
- * reductions.  Measured slower than the per-phase kernels on GB300 (94.6 vs
- * 39.4 us per iteration of one simulation when the launch takes an eighth of
- * the device, as it must for eight simulations to run side by side), because a
- * phase then runs several row items one after another per block.  The
+ * reductions.  Measured slower than the per-phase kernels on GB300: 57 vs 33 us
+ * per iteration of one sub-problem solve that has the device to itself (two
+ * blocks per SM, every phase behind a grid barrier), and more where the launch
+ * takes an eighth of the device, as it must for eight simulations to run side
+ * by side.  The
  * summation order of the dot products differs from the per-phase kernels (both
  * are deterministic).  Barrier waits are bounded (about two seconds); a
  * timeout ends the solve with PFF_ERR_BARRIER_TIMEOUT.  When the device cannot

@@ -789,7 +789,7 @@ static int pf_solve_group(Group& g, int max_pf, pff_problem* eh, bool& warmed) {
     launch_elem<T>(EL_PF_INIT, g.nx, g.ny, d, g.np, g.st);
     if constexpr (sizeof(T) == 4) {
         if (g_persist && !g.precond && g.np == 1 && g.nx == 512 && g.ny == 512 && !timing_on()) {
-            cudaError_t e = launch_persist_bccg((const Desc<float>*)g.d_desc, max_pf + 2,
+            cudaError_t e = launch_persist_bccg((const Desc<float>*)g.d_desc, max_pf,
                                                 persist_bccg_blocks(g_persist_share), g.st);
             if (e == cudaSuccess) {
                 if ((rc = poll<T>(g, true, eh))) return rc;
@@ -1510,7 +1510,7 @@ int pff_solve_phase_field(pff_problem* h, pff_step_report* out) {
         launch_elem<T>(EL_PF_INIT, h->nx, h->ny, d, 1, h->st);
         if constexpr (sizeof(T) == 4) {
             if (g_persist && !h->prm.pf_precondition && h->nx == 512 && h->ny == 512 && !timing_on()) {
-                cudaError_t e = launch_persist_bccg((const Desc<float>*)h->d_desc, p.pf_max_iter + 2,
+                cudaError_t e = launch_persist_bccg((const Desc<float>*)h->d_desc, p.pf_max_iter,
                                                     persist_bccg_blocks(1), h->st);
                 if (e == cudaSuccess) {
                     int r2 = poll<T>(g, true, h);

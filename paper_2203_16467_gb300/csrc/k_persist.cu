@@ -2,16 +2,16 @@
 // problem of 512 x 512 pixels per launch.
 //
 // The iterations of the phase-field sub-problem run inside one cooperative
-// launch whose blocks all stay resident.  The phases of an iteration -- the
-// direction and row FFT pass, the column Laplacian pass, the row-inverse pass
-// with J p and its dot products, the elementwise iterate with the residual
-// recurrence, and (when a value was clamped, every 32 iterations and to confirm
-// convergence) the explicit J v - b chain -- are the same device functions the
-// separate kernels use, separated by grid barriers that also carry the
+// launch whose blocks all stay resident.  They are the default path's slots (ops.cuh:
+// FPfSlotIn / FColLapPFS / FPfSlotOut), an iterate or an explicit J v - b each, by the same
+// device functions as the separate kernels, so the two differ only in the order
+// in which the dot products' block totals are summed.  The three phases of a slot are
+// separated by grid barriers that also carry the
 // reductions: each block reduces its share, the last block to arrive sums the
 // partials in a fixed order, runs the phase's finalizer (alpha, beta, the
 // stopping test) and releases the others.  No kernel boundary remains inside a
-// solve.
+// solve.  (One 512^2 solve with the device to itself: 57 us per iteration, the
+// separate kernels from captured graphs 33.)
 //
 // Every wait is bounded: a block that has not been released after about two
 // seconds of clock cycles sets status bit 8 and the abort flag and returns, and
@@ -167,15 +167,20 @@ __device__ __noinline__ bool row_fwd_phase(const Desc<float>& d, float2* work, c
 
 template <class OP>
 __device__ __noinline__ bool col_phase(const Desc<float>& d, float2* work, const float2* ctw, long long spin) {
-    const ModeK<float> mk(d);
+    constexpr int NR = ColNR<OP>::value;
+    ModeK<float> mk(d);
+    OP::mode_prep(d, mk);
+    Acc<float> acc[NR];
     for (int item = blockIdx.x; item < (d.nx / 2 + PB_CW) / PB_CW; item += gridDim.x) {   // mode columns only
         __syncthreads();
         float2 u[1][8];
         col512_load<float, 1, PB_CW>(d, item * PB_CW, u);
-        col512_item<float, 1, OP, PB_CW>(d, mk, item * PB_CW, work, ctw, u);
+        col512_item<float, 1, OP, PB_CW>(d, mk, item * PB_CW, work, ctw, u, acc);
     }
-    DF none[1];
-    return grid_sync<0>(d.ctrl, d.part, none, NoFin{}, spin);
+    DF v[NR];
+#pragma unroll
+    for (int k = 0; k < NR; ++k) v[k] = acc[k].df();
+    return grid_sync<NR>(d.ctrl, d.part, v, Fin<OP>{d}, spin);
 }
 
 template <class F>
@@ -192,21 +197,10 @@ __device__ __noinline__ bool row_inv_phase(const Desc<float>& d, float2* work, c
     return grid_sync<F::NR>(d.ctrl, d.part, v, Fin<F>{d}, spin);
 }
 
-template <class F>
-__device__ __noinline__ bool elem_phase(const Desc<float>& d, long long spin) {
-    const typename F::Ctx ctx = bcast_prep<F>(d);
-    Acc<float> acc[F::NR];
-    elem_items<float, F>(d, ctx, &acc[0]);
-    DF v[F::NR];
-#pragma unroll
-    for (int k = 0; k < F::NR; ++k) v[k] = acc[k].df();
-    return grid_sync<F::NR>(d.ctrl, d.part, v, Fin<F>{d}, spin);
-}
-
 constexpr int PB_WORK = RC::NSEQ * RC::SP > PB_CW * COL512_XS ? RC::NSEQ * RC::SP : PB_CW * COL512_XS;
 constexpr size_t PB_SMEM = (size_t)(RC::TWS + padded_len(512) + PB_WORK) * sizeof(float2);
 
-__global__ void __launch_bounds__(PB_NT, 4) k_bccg512(const Desc<float>* __restrict__ descs, int max_iters,
+__global__ void __launch_bounds__(PB_NT, 4) k_bccg512(const Desc<float>* __restrict__ descs, int max_slots,
                                                         long long spin) {
     const Desc<float>& d = descs[0];
     Ctrl* c = d.ctrl;
@@ -218,17 +212,11 @@ __global__ void __launch_bounds__(PB_NT, 4) k_bccg512(const Desc<float>* __restr
     stage_col512_twiddles<float>(d, ctw);
     cp_async_wait_all();
     __syncthreads();
-    for (int it = 0; it <= max_iters; ++it) {
+    for (int slot = 0; slot < max_slots; ++slot) {
         if (__ldcg(&c->pf_b) || ld_volatile(&c->bar_abort)) break;   // the same decision in every block
-        if (!row_fwd_phase<FPfA1<float>>(d, work, rtw, spin)) return;
-        if (!col_phase<FColLapPF>(d, work, ctw, spin)) return;
-        if (!row_inv_phase<FPfA3<float>>(d, work, rtw, spin)) return;
-        if (!elem_phase<FPfB1<float>>(d, spin)) return;
-        if (__ldcg(&c->pf_full)) {
-            if (!row_fwd_phase<FPfVIn<float>>(d, work, rtw, spin)) return;
-            if (!col_phase<FColLapPFFull>(d, work, ctw, spin)) return;
-            if (!row_inv_phase<FPfB3<float>>(d, work, rtw, spin)) return;
-        }
+        if (!row_fwd_phase<FPfSlotIn<float>>(d, work, rtw, spin)) return;
+        if (!col_phase<FColLapPFS>(d, work, ctw, spin)) return;
+        if (!row_inv_phase<FPfSlotOut<float>>(d, work, rtw, spin)) return;
     }
 }
 
@@ -261,11 +249,13 @@ long long barrier_spin_limit() {
     return spin > 0 ? spin : PB_SPIN_CYCLES;
 }
 
-// Launches the persistent solve of one FP32 512 x 512 problem (after its BCCG start).
+// Launches the persistent solve of one FP32 512 x 512 problem (after its BCCG start) of at most max_iters
+// iterations (its finalizers end it there).
 cudaError_t launch_persist_bccg(const Desc<float>* d, int max_iters, int blocks, cudaStream_t st) {
     if (blocks < 1) return cudaErrorInvalidConfiguration;
+    int max_slots = max_iters < (1 << 30) ? 2 * max_iters + 2 : 0x7fffffff;   // an iteration takes one or two
     long long spin = barrier_spin_limit();
-    void* args[] = {(void*)&d, (void*)&max_iters, (void*)&spin};
+    void* args[] = {(void*)&d, (void*)&max_slots, (void*)&spin};
     cudaError_t e = cudaLaunchCooperativeKernel((const void*)k_bccg512, dim3(blocks), dim3(PB_NT), args, PB_SMEM, st);
     count_launch();
     return e;
