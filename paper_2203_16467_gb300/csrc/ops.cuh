@@ -8,7 +8,7 @@
 // Newton residual (Eq. elasticity_nodal): FNewtonIn / FColGammaN / FNewtonOut.
 // Phase field (Algorithm 1): FPfInit, then one operator application per BCCG iteration and one more where
 // J v - b is evaluated explicitly, both by the same three kernels (FPfSlotIn / FColLapPFS / FPfSlotOut).
-// The preconditioned and the four-pass variants and the persistent kernel instead:
+// The preconditioned and the four-pass variants instead:
 //   A1 FPfA1 (p = -r + b p, masked) -> A2 lap -> A3 FPfA3 (p.Jp, r.p -> alpha)
 //   B1 FPfB1 (v = max(v + alpha p, v_con)) -> B2 lap -> B3 FPfB3 (r = Jv - b, active set,
 //   r.r, r.r_old -> beta, convergence).
@@ -698,7 +698,7 @@ struct FPfA3 {   // J p; p.Jp, r.p -> alpha = -(r.p)/(p.Jp)
 // come from sums of the iteration that forms r': sum a p'^2 = S1 - 2 beta S2 + beta^2 S3 and
 // r'.p' = -r'.r' + beta S4 with S1 = sum a r'^2, S2 = sum a r' p, S3 = sum a p^2 (free
 // pixels) and S4 = r'.p (pf_next_dir); the first direction p = -r from the start's sums.
-// (The preconditioned and four-pass variants and the persistent kernel keep FPfA1 / FColLapPF / FPfA3 /
+// (The preconditioned and four-pass variants keep FPfA1 / FColLapPF / FPfA3 /
 // FPfB1 and FPfVIn / FColLapPFFull / FPfB3 for the explicit residual.)
 struct FColLapPFQ {   // (as such the column pass of the cluster-resident solve)
     static constexpr int NR = 1;
