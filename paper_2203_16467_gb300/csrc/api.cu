@@ -792,10 +792,7 @@ static int pf_solve_group(Group& g, int max_pf, pff_problem* eh, bool& warmed) {
             cudaError_t e = launch_persist_bccg((const Desc<float>*)g.d_desc, max_pf,
                                                 persist_bccg_blocks(g_persist_share), g.st);
             if (e == cudaSuccess) {
-                if ((rc = poll<T>(g, true, eh))) return rc;
-                if (g.h_ctrl[0].status & 8)
-                    return fail(eh, PFF_ERR_BARRIER_TIMEOUT, "persistent phase-field solve: a grid barrier timed out");
-                launch_elem<T>(EL_POST, g.nx, g.ny, d, g.np, g.st);
+                launch_elem<T>(EL_POST, g.nx, g.ny, d, g.np, g.st);   // (given up: leaves phi)
                 return 0;
             }
             cudaGetLastError();   // not launched (e.g. not enough resident capacity): chunked path
@@ -1512,13 +1509,7 @@ int pff_solve_phase_field(pff_problem* h, pff_step_report* out) {
             if (g_persist && !h->prm.pf_precondition && h->nx == 512 && h->ny == 512 && !timing_on()) {
                 cudaError_t e = launch_persist_bccg((const Desc<float>*)h->d_desc, p.pf_max_iter,
                                                     persist_bccg_blocks(1), h->st);
-                if (e == cudaSuccess) {
-                    int r2 = poll<T>(g, true, h);
-                    if (r2) return r2;
-                    if (g.h_ctrl[0].status & 8)
-                        return fail(h, PFF_ERR_BARRIER_TIMEOUT, "persistent phase-field solve: a grid barrier timed out");
-                    return finish();
-                }
+                if (e == cudaSuccess) return finish();
                 cudaGetLastError();
             }
         }

@@ -1,4 +1,5 @@
-"""The one-launch solves of small FP32 grids when a wait between their blocks runs out: a limit of one
+"""The one-launch solves of small FP32 grids (and the persistent one of 512^2 in steps and batches) when a
+wait between their blocks runs out: a limit of one
 cycle ends the first wait for which the bytes are not there yet.  The calls report
 PFF_ERR_BARRIER_TIMEOUT, apply nothing of the given-up solve, and the handle then solves as a fresh
 one does.  The sizes have CTAs with and without mode columns, one and several rows per warp."""
@@ -127,3 +128,40 @@ def test_laplacian_leaves_nan(pff, nx, ny):
     lap(z)
     assert torch.isnan(y).all()
     assert torch.isfinite(z).all() and z.abs().max() > 0
+
+
+def test_persistent_step_and_batch(pff):
+    import torch
+    n = 512
+    try:
+        pff.set_persistent(True)
+        p = make(pff, n, n)
+        before = p.get_fields(pff.FIELD_PHI)
+        done = ctypes.c_int(7)
+        pff.set_barrier_spin_limit(1)
+        rc = pff.lib.pff_step_load(p.h, 2, (pff.StepReport * 2)(), ctypes.byref(done))
+        pff.set_barrier_spin_limit(0)
+        assert rc == pff.ERR_BARRIER_TIMEOUT and done.value == 0
+        np.testing.assert_array_equal(p.get_fields(pff.FIELD_PHI), before)
+        assert len(p.step_load(1)) == 1
+        # a batch with a small grid of FP64 beside it, whose solves have no such waits: its step counts
+        small = pff.Problem(32, 32, pff.FP64, params=dict(nu=0.2, ell=ELL))
+        small.set_strain(None, (0.0, 1.0, 0.0))
+        b = pff.create_batch(2, pff.problem_bytes(n, n, pff.MIXED) + pff.problem_bytes(32, 32, pff.FP64),
+                             torch.cuda.Stream().cuda_stream)
+        for x in (p, small):
+            pff.batch_admit(b, x.h)
+        before = p.get_fields(pff.FIELD_PHI)
+        reps, done = (pff.StepReport * 4)(), (ctypes.c_int * 2)(7, 7)
+        pff.set_barrier_spin_limit(1)
+        rc = pff.lib.pff_batch_step(b, 2, reps, done)
+        pff.set_barrier_spin_limit(0)
+        assert rc == pff.ERR_BARRIER_TIMEOUT and list(done) == [0, 1]
+        assert reps[0].status == pff.ERR_BARRIER_TIMEOUT and reps[2].status == pff.OK and reps[2].bccg_iters > 0
+        np.testing.assert_array_equal(p.get_fields(pff.FIELD_PHI), before)
+        pff.destroy_batch(b)
+        p.close()
+        small.close()
+    finally:
+        pff.set_barrier_spin_limit(0)
+        pff.set_persistent(False)
